@@ -1155,6 +1155,7 @@ struct FaceVariant {
     // interior tiles stage their box from tensor-map copies (FP32 2D with a scratch level;
     // the copies land in the corrector's scratch before the corrector uses it)
     static constexpr bool TMA = TMA_;
+    static constexpr bool LANES = false;   // true: the lane kernel of pond_face2.cuh
 };
 
 // Instantiations (MODE): FACE_PLAIN; FACE_COLLECT also writes (features, converged frame)

@@ -11,6 +11,7 @@
 #include <cstdio>
 
 #include "pond_batch.cuh"
+#include "pond_face2.cuh"
 
 namespace pond {
 
@@ -21,19 +22,20 @@ struct VList {
 
 // ---------------------------------------------------------------- face kernel
 
+// D2Q16: the lane kernel (pond_face2.cuh) in tiles that keep whole warps on one direction; us a
+// launch on the 1024^2 quadrants in FP32: 16 x 8 / 3 CTAs per SM 290, 32 x 4 / 3 302, 16 x 8 / 2 318 (the
+// 1001 x 253 interface: 110, 107, 117), against 328-380 for the node-by-node tiles kept below for
+// comparison; FP64 256^2: 8 x 4 / 4 1314, 8 x 8 / 2 1362, 16 x 4 / 2 1401.
 template <int D, typename R>
 struct FaceList;
 template <>
 struct FaceList<2, float> {
-    using type = VList<FaceVariant<2, 32, 4, 2>, FaceVariant<2, 16, 8, 2>, FaceVariant<2, 64, 2, 2>,
-                       FaceVariant<2, 16, 4, 4>, FaceVariant<2, 32, 4, 1>, FaceVariant<2, 16, 8, 3>,
-                       FaceVariant<2, 16, 4, 6>, FaceVariant<2, 8, 8, 4>, FaceVariant<2, 8, 8, 4, 1>,
-                       FaceVariant<2, 8, 8, 4, 2>, FaceVariant<2, 16, 4, 4, 2>, FaceVariant<2, 8, 8, 4, 1, true>,
-                       FaceVariant<2, 8, 8, 3, 1, true>, FaceVariant<2, 8, 8, 4, 2, true>>;
+    using type = VList<LaneVariant<16, 8, 3>, LaneVariant<32, 4, 3>, LaneVariant<16, 8, 2>, FaceVariant<2, 8, 8, 4>,
+                       FaceVariant<2, 8, 8, 4, 1>, FaceVariant<2, 8, 8, 4, 2>, FaceVariant<2, 8, 8, 4, 1, true>, FaceVariant<2, 8, 8, 4, 2, true>>;
 };
 template <>
 struct FaceList<2, double> {
-    using type = VList<FaceVariant<2, 32, 4, 1>, FaceVariant<2, 16, 8, 1>, FaceVariant<2, 16, 4, 2>, FaceVariant<2, 8, 8, 2>>;
+    using type = VList<LaneVariant<8, 4, 4>, LaneVariant<8, 8, 2>, LaneVariant<16, 4, 2>>;
 };
 template <typename R>
 struct FaceList<1, R> {
@@ -45,7 +47,10 @@ template <int D, typename R, typename V, typename... Rest>
 void face_name_at(int v, char *buf, size_t n)
 {
     if (v <= 0 || sizeof...(Rest) == 0) {
-        if (D == 2)
+        if constexpr (V::LANES)
+            std::snprintf(buf, n, "face %dx%d cells, %d threads, %d CTA/SM, by upwind side%s", V::TX, V::TY,
+                          lane_threads<R, V>(), V::MINB, VecOf<R>::lanes > 1 ? ", two faces a thread" : "");
+        else if constexpr (D == 2)
             std::snprintf(buf, n, "face %dx%d cells, %d threads, %d CTA/SM%s%s", V::TX, V::TY, V::THREADS, V::MINB,
                           V::SCR == 1 ? ", centre cells in shared scratch"
                                       : V::SCR == 2 ? ", centre cells and moment sums in shared scratch" : "",

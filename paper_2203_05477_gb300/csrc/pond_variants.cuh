@@ -11,6 +11,11 @@ template <int D, typename R, int MODE, typename V>
 void launch_face_one(const Params<D, R> &P, cudaStream_t st)
 {
     const dim3 g(unsigned((P.nx + 1 + V::TX - 1) / V::TX), D == 2 ? unsigned((P.ny + 1 + V::TY - 1) / V::TY) : 1u);
+    if constexpr (V::LANES) {
+        constexpr int bytes = int(lane_smem_bytes<R, V>());
+        cudaFuncSetAttribute(lane_face_kernel<R, MODE, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        lane_face_kernel<R, MODE, V><<<g, lane_threads<R, V>(), bytes, st>>>(P);
+    } else {
     if constexpr (V::TMA) {
         // the tensor maps of the buffer that holds the state now; without them (a grid whose
         // rows are not 16-byte multiples) the same tile stages every cell per thread
@@ -23,6 +28,7 @@ void launch_face_one(const Params<D, R> &P, cudaStream_t st)
         }
     }
     face_kernel<D, R, MODE, V><<<g, V::THREADS, 0, st>>>(P);
+    }
 }
 
 template <int D, typename R, int MODE, typename V, typename... Rest>
