@@ -133,9 +133,13 @@ void launch_step_fused(int v, const Params<D, R> &P, cudaStream_t st);
 
 // ---------------------------------------------------------------- cell kernel
 
-constexpr int kCellBlocks[9] = {256, 128, 512, 256, 256, 128, 32, 128, 128};
-constexpr int kCellMinBlocks[9] = {1, 1, 1, 3, 4, 6, 1, 3, 1};   // CTAs per SM asked of the register allocator
-constexpr bool kCellGridStride[9] = {false, false, false, false, false, false, false, true, true};
+// Entry 0, the default, is the grid-stride kernel at 128 threads and 3 CTAs per SM: the fastest or
+// within 2% of it from 200 cells to 4 M (us a launch, against the plain 256-thread one: FP32
+// quadrants 1024^2 93 / 133, tube of 4 M cells 120 / 132; FP64 quadrants 256^2 114 / 116, tube of
+// 400 cells 23 / 31).
+constexpr int kCellBlocks[9] = {128, 128, 512, 256, 256, 128, 32, 256, 128};
+constexpr int kCellMinBlocks[9] = {3, 1, 1, 3, 4, 6, 1, 1, 1};   // CTAs per SM asked of the register allocator
+constexpr bool kCellGridStride[9] = {true, false, false, false, false, false, false, false, true};
 constexpr int kCellVariants = 9;
 
 template <int D, typename R>

@@ -72,7 +72,7 @@ void launch_cell(int v, const Params<D, R> &P, cudaStream_t st)
         return unsigned(need < cap ? need : cap);
     };
     switch (v) {
-    case 7: cell_kernel<D, R, 128, 3, false, true><<<gs_blocks(128), 128, 0, st>>>(P); break;
+    case 7: cell_kernel<D, R, 256><<<blocks(256), 256, 0, st>>>(P); break;
     case 8: cell_kernel<D, R, 128, 1, false, true><<<gs_blocks(128), 128, 0, st>>>(P); break;
     case 1: cell_kernel<D, R, 128><<<blocks(128), 128, 0, st>>>(P); break;
     case 2: cell_kernel<D, R, 512><<<blocks(512), 512, 0, st>>>(P); break;
@@ -80,7 +80,7 @@ void launch_cell(int v, const Params<D, R> &P, cudaStream_t st)
     case 4: cell_kernel<D, R, 256, 4><<<blocks(256), 256, 0, st>>>(P); break;
     case 5: cell_kernel<D, R, 128, 6><<<blocks(128), 128, 0, st>>>(P); break;
     case 6: cell_kernel<D, R, 32><<<blocks(32), 32, 0, st>>>(P); break;
-    default: cell_kernel<D, R, 256><<<blocks(256), 256, 0, st>>>(P); break;
+    default: cell_kernel<D, R, 128, 3, false, true><<<gs_blocks(128), 128, 0, st>>>(P); break;
     }
 }
 
