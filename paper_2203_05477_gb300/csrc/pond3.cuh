@@ -40,31 +40,13 @@ struct NC3 {
 };
 constexpr int kNF3 = NC3<3>::value, kNG3 = NC3<2>::value, kNFS3 = kNF3 - 3;
 
-// orders (r, s, t) of packed index k
-__host__ __device__ constexpr int h3r(int k)
-{
-    for (int r = 0; r <= 3; ++r)
-        for (int s = 0; r + s <= 3; ++s)
-            for (int t = 0; r + s + t <= 3; ++t)
-                if (h3idx(r, s, t) == k) return r;
-    return 0;
-}
-__host__ __device__ constexpr int h3s(int k)
-{
-    for (int r = 0; r <= 3; ++r)
-        for (int s = 0; r + s <= 3; ++s)
-            for (int t = 0; r + s + t <= 3; ++t)
-                if (h3idx(r, s, t) == k) return s;
-    return 0;
-}
-__host__ __device__ constexpr int h3t(int k)
-{
-    for (int r = 0; r <= 3; ++r)
-        for (int s = 0; r + s <= 3; ++s)
-            for (int t = 0; r + s + t <= 3; ++t)
-                if (h3idx(r, s, t) == k) return t;
-    return 0;
-}
+// orders (r, s, t) of packed index k, in closed form (block n = r + s + t, then j = s + t, then t)
+__host__ __device__ constexpr int h3n(int k) { return (k >= 1) + (k >= 4) + (k >= 10); }
+__host__ __device__ constexpr int h3rem(int k) { return k - h3n(k) * (h3n(k) + 1) * (h3n(k) + 2) / 6; }
+__host__ __device__ constexpr int h3j(int k) { return (h3rem(k) >= 1) + (h3rem(k) >= 3) + (h3rem(k) >= 6); }
+__host__ __device__ constexpr int h3t(int k) { return h3rem(k) - h3j(k) * (h3j(k) + 1) / 2; }
+__host__ __device__ constexpr int h3s(int k) { return h3j(k) - h3t(k); }
+__host__ __device__ constexpr int h3r(int k) { return h3n(k) - h3j(k); }
 
 // stored f plane of coefficient k (-1: a first-order one, zero in the cell's own frame)
 __host__ __device__ constexpr int fplane3(int k) { return k == 0 ? 0 : (k <= 3 ? -1 : k - 3); }
@@ -117,8 +99,7 @@ __device__ __forceinline__ void shift_scale_3d(const R *in, const Map1<R> &X, co
 
 // Faces work in face axes (normal, first tangential, second tangential), the tangential
 // axes being the other two in increasing order: x-face (x, y, z), y-face (y, x, z),
-// z-face (z, x, y).  lab axis of face axis q:
-__host__ __device__ __forceinline__ int face_axis(int dir, int q) { return q == 0 ? dir : (q == 1 ? (dir == 0 ? 1 : 0) : (dir == 2 ? 1 : 2)); }
+// z-face (z, x, y).
 // lab index of face-axis orders (r, s, t)
 __host__ __device__ __forceinline__ int lab_of_face(int dir, int r, int s, int t)
 {
@@ -140,28 +121,12 @@ __host__ __device__ constexpr FacePerm make_face_perm()
 }
 static __constant__ FacePerm kFacePerm = make_face_perm();
 
-// the first NC3<N> coefficients of a staged cell in face axes (total orders are kept, so the
-// g set (N = 2) is the head of the same permutation)
-template <int N, typename R>
-__device__ __forceinline__ void to_face(const R *lab, R *face, int dir)
-{
-#pragma unroll
-    for (int k = 0; k < NC3<N>::value; ++k) face[k] = lab[kFacePerm.k[dir][k]];
-}
-// face-axis coefficients back to lab axes, by selects (the destination is a register array)
-template <int N, typename R>
-__device__ __forceinline__ void from_face(const R *face, R *lab, int dir)
-{
-#pragma unroll
-    for (int r = 0; r <= N; ++r)
-#pragma unroll
-        for (int s = 0; r + s <= N; ++s)
-#pragma unroll
-            for (int t = 0; r + s + t <= N; ++t)
-                lab[h3idx(r, s, t)] = dir == 0 ? face[h3idx(r, s, t)] : (dir == 1 ? face[h3idx(s, r, t)] : face[h3idx(t, r, s)]);
-}
-
 // ------------------------------------------------------------------ parameters
+
+// faces listed in this step, the next one to take, and the tail's CTAs that are through
+struct TailList {
+    unsigned int n, next, ctas, pad;
+};
 
 template <typename R>
 struct Params3 {
@@ -180,6 +145,11 @@ struct Params3 {
     W *ffr[3];                        // [4][nf]
     Clock *clock;
     Diag *diag;
+    // list of the faces that the face kernel leaves to its tail (room for every face)
+    TailList *tail;
+    unsigned long long *tail_items;
+    int tail_at;                      // a warp with at most this many unfinished faces lists them
+    int sms;                          // SMs of the device (grid of the tail kernel)
     __host__ __device__ long long ncell() const { return nx * ny * nz; }
     __host__ __device__ long long nf(int a) const
     {
@@ -227,7 +197,6 @@ struct StagedCell3 {
     R B[kNG3];
     R du[3];   // frame velocity relative to the tile reference (lab axes)
     R T;
-    R pad;     // odd size in words: neighbouring threads' cells fall in distinct banks
 };
 
 template <typename R>
@@ -280,561 +249,6 @@ __device__ __forceinline__ void load_cell3(const Params3<R> &P, long long i, lon
 #pragma unroll
     for (int q = 1; q < kNG3; ++q) c.B[q] = cp * c.B[q];
     c.T = T;
-}
-
-// ------------------------------------------------------------------ face corrector
-
-// Stencil slots of a face (as in the oracle): 0 LL, 1 L, 2 R, 3 RR along the normal; 4 L-,
-// 5 L+, 6 R-, 7 R+ along the first tangential axis; 8 L-, 9 L+, 10 R-, 11 R+ along the
-// second.  Offsets in face axes from cell R (normal, first tangential, second tangential).
-__device__ __forceinline__ void slot_offset(int s, int &on, int &o1, int &o2)
-{
-    if (s < 4) {
-        on = s - 2;
-        o1 = 0;
-        o2 = 0;
-    } else {
-        const int side = ((s - 4) & 3) >> 1;   // 0: L, 1: R
-        const int sg = (s & 1) ? 1 : -1;
-        on = side - 1;
-        o1 = s < 8 ? sg : 0;
-        o2 = s < 8 ? 0 : sg;
-    }
-}
-
-// the staged box of a CTA and the face's place in it
-template <typename R>
-struct FaceBox {
-    const StagedCell3<R> *tile;
-    int BX, BY;          // box extents along x and y (lab)
-    int bx, by, bz;      // box coordinates of cell R of the face
-    int dir;
-    __device__ __forceinline__ const StagedCell3<R> *slot(int s) const
-    {
-        int on, o1, o2;
-        slot_offset(s, on, o1, o2);
-        // lab offsets by selects (no run-time indexed array)
-        const int a1 = face_axis(dir, 1), a2 = face_axis(dir, 2);
-        const int ox = (dir == 0 ? on : 0) + (a1 == 0 ? o1 : 0) + (a2 == 0 ? o2 : 0);
-        const int oy = (dir == 1 ? on : 0) + (a1 == 1 ? o1 : 0) + (a2 == 1 ? o2 : 0);
-        const int oz = (dir == 2 ? on : 0) + (a1 == 2 ? o1 : 0) + (a2 == 2 ? o2 : 0);
-        return &tile[((bz + oz) * BY + (by + oy)) * BX + (bx + ox)];
-    }
-};
-
-// frame maps of a staged cell into the pass frame, in face axes: s = sqrt(Tc/Tl),
-// e = s^2 - 1, d = (uc - ul)/sqrt(Tl)
-template <typename R>
-__device__ __forceinline__ void cell_maps3(const StagedCell3<R> *c, int dir, const R *dref, const R *dl, R Tl, R invTl,
-                                           R rsqTl, Map1<R> &X, Map1<R> &Y, Map1<R> &Z)
-{
-    const R s = sqrt(c->T * invTl);
-    const R e = (c->T - Tl) * invTl;
-    X = Map1<R>(s, e, (c->du[face_axis(dir, 0)] - dref[0] - dl[0]) * rsqTl);
-    Y = Map1<R>(s, e, (c->du[face_axis(dir, 1)] - dref[1] - dl[1]) * rsqTl);
-    Z = Map1<R>(s, e, (c->du[face_axis(dir, 2)] - dref[2] - dl[2]) * rsqTl);
-}
-
-// One corrector pass at a face (Sec. III.B.3) in frame (dl, Tl) (velocity relative to the
-// face reference dref, face axes).  A population (m, n, p) is reconstructed as
-// u + off_n lim(u - l, h - u) + off_1 lim(u - t1-, t1+ - u) + off_2 lim(u - t2-, t2+ - u)
-// from its upwind cell u, that cell's normal neighbours l, h and its tangential neighbours,
-// and only the moments of the reconstructions are kept; they are linear in the three terms,
-// so each normal node m runs three sweeps (normal, first and second tangential slope), each
-// needing the upwind cell and two neighbours.  The cells are re-expressed in the pass frame,
-// collapsed along the normal at c_m and kept in a per-thread shared-memory scratch (3 slots
-// of 16 values, slot-major, thread-minor over NT threads).  Phi: moments of f (order 3),
-// Psi: of g (order 2), face axes.
-template <typename R>
-__device__ __forceinline__ void collapse_normal(const StagedCell3<R> *c, int dir, const R *dref, const R *dl, R Tl,
-                                                R invTl, R rsqTl, const R *hn, R *slot, int NT)
-{
-    Map1<R> X(R(1), R(0), R(0)), Y = X, Z = X;
-    cell_maps3<R>(c, dir, dref, dl, Tl, invTl, rsqTl, X, Y, Z);
-    R tmp[kNF3], F[kNF3];
-    to_face<3, R>(c->A, tmp, dir);
-    shift_scale_3d<3, R, true>(tmp, X, Y, Z, F);   // staged f: zero first order
-#pragma unroll
-    for (int s2 = 0; s2 <= 3; ++s2)
-#pragma unroll
-        for (int t2 = 0; s2 + t2 <= 3; ++t2) {
-            R acc = R(0);
-#pragma unroll
-            for (int r = 0; r + s2 + t2 <= 3; ++r) acc += F[h3idx(r, s2, t2)] * hn[r];
-            slot[h2st(s2, t2) * NT] = acc;
-        }
-    R tg[kNG3], G[kNG3];
-    to_face<2, R>(c->B, tg, dir);
-    shift_scale_3d<2, R>(tg, X, Y, Z, G);
-#pragma unroll
-    for (int s2 = 0; s2 <= 2; ++s2)
-#pragma unroll
-        for (int t2 = 0; s2 + t2 <= 2; ++t2) {
-            R acc = R(0);
-#pragma unroll
-            for (int r = 0; r + s2 + t2 <= 2; ++r) acc += G[h3idx(r, s2, t2)] * hn[r];
-            slot[(10 + h2st(s2, t2)) * NT] = acc;
-        }
-}
-
-// The populations (n, p = 0..3) of one sweep at normal node m, FP32: the three scratch slots
-// (upwind cell, two neighbours; normal-collapsed) collapsed along the first tangential axis
-// at c_n, evaluated at c_p, reconstructed (plain * upwind + off * limited slope) and their
-// moments along the second tangential axis accumulated into S1f (f, orders 0..3) and S1g
-// (g, 0..2).  f rides in lane x and g in lane y of FP32x2 pairs for the orders 0..2.
-__device__ __forceinline__ void sweep_node_f32(const float *scr, int NT, int n, float off1, bool off_by_p, float plain,
-                                               float sqTl, float u2, float h_d2, int limiter, float *S1f, float *S1g)
-{
-    const NodeTab<float> &tab = node_tab<float>();
-    const float h0 = tab.hen[n][0], h1 = tab.hen[n][1], h2 = tab.hen[n][2], h3 = tab.hen[n][3];
-    const float2 H0 = bc2(h0), H1 = bc2(h1), H2 = bc2(h2);
-    // c[q][t2]: lane x f, lane y g (t2 = 0..2); cf3[q]: f at t2 = 3
-    float2 c[3][3];
-    float cf3[3];
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        const float *b = scr + q * 16 * NT;
-        auto F = [&](int s2, int t2) { return b[h2st(s2, t2) * NT]; };
-        auto G = [&](int s2, int t2) { return b[(10 + h2st(s2, t2)) * NT]; };
-        // t2 = 0: f sums s2 = 0..3, g s2 = 0..2
-        float2 a0 = __fmul2_rn(make_float2(F(0, 0), G(0, 0)), H0);
-        a0 = __ffma2_rn(make_float2(F(1, 0), G(1, 0)), H1, a0);
-        a0 = __ffma2_rn(make_float2(F(2, 0), G(2, 0)), H2, a0);
-        a0.x += F(3, 0) * h3;
-        // t2 = 1: f s2 = 0..2, g s2 = 0..1
-        float2 a1 = __fmul2_rn(make_float2(F(0, 1), G(0, 1)), H0);
-        a1 = __ffma2_rn(make_float2(F(1, 1), G(1, 1)), H1, a1);
-        a1.x += F(2, 1) * h2;
-        // t2 = 2: f s2 = 0..1, g s2 = 0
-        float2 a2 = __fmul2_rn(make_float2(F(0, 2), G(0, 2)), H0);
-        a2.x += F(1, 2) * h1;
-        c[q][0] = a0;
-        c[q][1] = a1;
-        c[q][2] = a2;
-        cf3[q] = F(0, 3) * h0;
-    }
-    float2 S[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-    float S3 = 0.f;
-    const float2 minus1 = bc2(-1.f);
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-        const float off = off_by_p ? -(sqTl * float(node_c(p)) + u2) * h_d2 : off1;
-        float2 v[3];
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            float2 a = __fmul2_rn(c[q][0], bc2(float(hen(0, p))));
-            a = __ffma2_rn(c[q][1], bc2(float(hen(1, p))), a);
-            a = __ffma2_rn(c[q][2], bc2(float(hen(2, p))), a);
-            a.x += cf3[q] * float(hen(3, p));
-            v[q] = a;
-        }
-        const float2 lim = limit2(limiter, __ffma2_rn(v[1], minus1, v[0]), __ffma2_rn(v[0], minus1, v[2]));
-        const float2 b = __ffma2_rn(bc2(off), lim, __fmul2_rn(bc2(plain), v[0]));
-#pragma unroll
-        for (int t2 = 0; t2 <= 2; ++t2) S[t2] = __ffma2_rn(bc2(float(node_w(p) * he(t2, p))), b, S[t2]);
-        S3 += float(node_w(p) * he(3, p)) * b.x;
-    }
-#pragma unroll
-    for (int t2 = 0; t2 <= 2; ++t2) {
-        S1f[t2] = S[t2].x;
-        S1g[t2] = S[t2].y;
-    }
-    S1f[3] = S3;
-}
-
-template <typename R, int NT>
-__device__ __forceinline__ void corrector_pass3(const FaceBox<R> &box, const R *dref, const R *uabs, const R *dl, R Tl,
-                                                R h_dn, R h_d1, R h_d2, int limiter, R *scr, R *Phi, R *Psi)
-{
-    const R invTl = R(1) / Tl;
-    const R rsqTl = sqrt(invTl);
-    const R sqTl = Tl * rsqTl;
-    const NodeTab<R> &tab = node_tab<R>();
-#pragma unroll
-    for (int q = 0; q < kNF3; ++q) Phi[q] = R(0);
-#pragma unroll
-    for (int q = 0; q < kNG3; ++q) Psi[q] = R(0);
-    const R un = uabs[0] + dl[0], u1 = uabs[1] + dl[1], u2 = uabs[2] + dl[2];
-#pragma unroll 1
-    for (int m = 0; m < 4; ++m) {
-        const R vn = sqTl * tab.c[m] + un;
-        const bool left = vn > R(0);
-        const R offn = (left ? R(0.5) : R(-0.5)) - vn * h_dn;
-        const R hn[4] = {tab.hen[m][0], tab.hen[m][1], tab.hen[m][2], tab.hen[m][3]};
-        // scratch slot 0: the upwind cell
-        collapse_normal<R>(box.slot(left ? 1 : 2), box.dir, dref, dl, Tl, invTl, rsqTl, hn, scr, NT);
-        // moments over the tangential nodes of this normal node, in (s, t)
-        R S2f[10], S2g[6];
-#pragma unroll
-        for (int q = 0; q < 10; ++q) S2f[q] = R(0);
-#pragma unroll
-        for (int q = 0; q < 6; ++q) S2g[q] = R(0);
-#pragma unroll 1
-        for (int sw = 0; sw < 3; ++sw) {
-            // the two neighbours of the sweep: normal (l, h), then first and second tangential (-, +)
-            const int sa = sw == 0 ? (left ? 0 : 1) : (left ? 4 : 6) + 4 * (sw - 1);
-            const int sb = sw == 0 ? (left ? 2 : 3) : sa + 1;
-            collapse_normal<R>(box.slot(sa), box.dir, dref, dl, Tl, invTl, rsqTl, hn, scr + 16 * NT, NT);
-            collapse_normal<R>(box.slot(sb), box.dir, dref, dl, Tl, invTl, rsqTl, hn, scr + 32 * NT, NT);
-            const R plain = sw == 0 ? R(1) : R(0);
-#pragma unroll 1
-            for (int n = 0; n < 4; ++n) {
-                const R off1 = sw == 0 ? offn : -(sqTl * tab.c[n] + u1) * h_d1;
-                R S1f[4] = {R(0), R(0), R(0), R(0)}, S1g[3] = {R(0), R(0), R(0)};
-                if constexpr (sizeof(R) == 4) {
-                    // FP32: f in lane x and g in lane y of FP32x2 pairs for the orders both carry
-                    // (0..2), f's third order alone
-                    sweep_node_f32(scr, NT, n, off1, sw == 2, plain, sqTl, u2, h_d2, limiter, S1f, S1g);
-                } else {
-                // collapse the three slots along the first tangential axis at c_n
-                R cf[3][4], cg[3][3];
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-#pragma unroll
-                    for (int t2 = 0; t2 <= 3; ++t2) {
-                        R acc = R(0);
-#pragma unroll
-                        for (int s2 = 0; s2 + t2 <= 3; ++s2) acc += scr[(q * 16 + h2st(s2, t2)) * NT] * tab.hen[n][s2];
-                        cf[q][t2] = acc;
-                    }
-#pragma unroll
-                    for (int t2 = 0; t2 <= 2; ++t2) {
-                        R acc = R(0);
-#pragma unroll
-                        for (int s2 = 0; s2 + t2 <= 2; ++s2) acc += scr[(q * 16 + 10 + h2st(s2, t2)) * NT] * tab.hen[n][s2];
-                        cg[q][t2] = acc;
-                    }
-                }
-#pragma unroll
-                for (int p = 0; p < 4; ++p) {
-                    const R off = sw == 2 ? -(sqTl * R(node_c(p)) + u2) * h_d2 : off1;
-                    R fv[3], gv[3];
-#pragma unroll
-                    for (int q = 0; q < 3; ++q) {
-                        R a = R(0), b = R(0);
-#pragma unroll
-                        for (int t2 = 0; t2 <= 3; ++t2) a += cf[q][t2] * R(hen(t2, p));
-#pragma unroll
-                        for (int t2 = 0; t2 <= 2; ++t2) b += cg[q][t2] * R(hen(t2, p));
-                        fv[q] = a;
-                        gv[q] = b;
-                    }
-                    const R fb = plain * fv[0] + off * limit<R>(limiter, fv[0] - fv[1], fv[2] - fv[0]);
-                    const R gb = plain * gv[0] + off * limit<R>(limiter, gv[0] - gv[1], gv[2] - gv[0]);
-#pragma unroll
-                    for (int t2 = 0; t2 <= 3; ++t2) S1f[t2] += R(node_w(p) * he(t2, p)) * fb;
-#pragma unroll
-                    for (int t2 = 0; t2 <= 2; ++t2) S1g[t2] += R(node_w(p) * he(t2, p)) * gb;
-                }
-                }
-#pragma unroll
-                for (int s2 = 0; s2 <= 3; ++s2)
-#pragma unroll
-                    for (int t2 = 0; s2 + t2 <= 3; ++t2) S2f[h2st(s2, t2)] += tab.whe[n][s2] * S1f[t2];
-#pragma unroll
-                for (int s2 = 0; s2 <= 2; ++s2)
-#pragma unroll
-                    for (int t2 = 0; s2 + t2 <= 2; ++t2) S2g[h2st(s2, t2)] += tab.whe[n][s2] * S1g[t2];
-            }
-        }
-#pragma unroll
-        for (int r = 0; r <= 3; ++r)
-#pragma unroll
-            for (int s2 = 0; r + s2 <= 3; ++s2)
-#pragma unroll
-                for (int t2 = 0; r + s2 + t2 <= 3; ++t2) Phi[h3idx(r, s2, t2)] += tab.whe[m][r] * S2f[h2st(s2, t2)];
-#pragma unroll
-        for (int r = 0; r <= 2; ++r)
-#pragma unroll
-            for (int s2 = 0; r + s2 <= 2; ++s2)
-#pragma unroll
-                for (int t2 = 0; r + s2 + t2 <= 2; ++t2) Psi[h3idx(r, s2, t2)] += tab.whe[m][r] * S2g[h2st(s2, t2)];
-    }
-}
-
-// frame of a pass's moments relative to the pass frame (face axes): rho, du, T
-template <typename R>
-__device__ __forceinline__ bool pass_frame3(const R *Phi, const R *Psi, R Tl, R Cv, R &rho, R *du, R &T)
-{
-    rho = Phi[0];
-    const R sq = sqrt(Tl);
-    du[0] = sq * Phi[h3idx(1, 0, 0)] / rho;
-    du[1] = sq * Phi[h3idx(0, 1, 0)] / rho;
-    du[2] = sq * Phi[h3idx(0, 0, 1)] / rho;
-    const R k2 = du[0] * du[0] + du[1] * du[1] + du[2] * du[2];
-    const R tr = Phi[h3idx(2, 0, 0)] + Phi[h3idx(0, 2, 0)] + Phi[h3idx(0, 0, 2)] + R(3) * Phi[0];
-    T = (R(0.5) * Tl * tr + Psi[0] - R(0.5) * rho * k2) / (Cv * rho);
-    return T > R(0) && isfinite(T) && isfinite(rho) && isfinite(du[0]) && isfinite(du[1]) && isfinite(du[2]);
-}
-
-template <typename R>
-struct FaceOut3 {
-    R F[kNF3];   // face populations' coefficients in the face frame (lab axes)
-    R G[kNG3];
-    R du[3];     // face frame velocity minus the predictor's (lab axes)
-    R T;
-    int iters, fallbacks;
-    bool done, have;
-};
-
-// The predictor-corrector of one face (the readings of the D2Q16 kernel: convergence rule,
-// restart once from the pooled moments of the stencil, the last valid pass's moments
-// Grad-projected into the frame they define, then Eq. FluxTransf).
-constexpr int kKeep3 = 3 * 16;   // first scratch slot of the kept frames (after the corrector's)
-
-template <typename R, int NT>
-__device__ __forceinline__ void solve_face3(const FaceBox<R> &box, const R *dref, const R *uabs, R Tpred, R h_dn, R h_d1,
-                                            R h_d2, R Cv, R tol, R wb, R we, int limiter, int max_iter, int fixed_iters,
-                                            R *scr, FaceOut3<R> &o)
-{
-    R dl[3] = {R(0), R(0), R(0)}, Tl = Tpred;
-    // the last valid pass's frames (its frame dl, Tl, and the frame its moments define: du,
-    // T1, rho1) wait in the thread's scratch after the corrector's 3 x 16 values, read and
-    // written with volatile accesses, instead of staying live in registers across the passes
-    auto kput = [&](int q, R v) { *reinterpret_cast<volatile R *>(&scr[(kKeep3 + q) * NT]) = v; };
-    auto kget = [&](int q) -> R { return *reinterpret_cast<volatile R *>(&scr[(kKeep3 + q) * NT]); };
-    bool have = false, done = false, restarted = false, last_valid = false, recompute = false;
-    int iters = 0;
-    o.fallbacks = 0;
-    R Phi[kNF3], Psi[kNG3];
-    // one call site of the pass: the last iteration of this loop recomputes the last valid
-    // pass when the final one defined no frame
-    for (int k = 0;; ++k) {
-        const bool run = recompute || (k < max_iter && !done);
-        if (!run) {
-            if (have && !last_valid) {
-                recompute = true;
-                continue;
-            }
-            break;
-        }
-        R dlp[3] = {dl[0], dl[1], dl[2]}, Tlp = Tl;
-        if (recompute) {
-#pragma unroll
-            for (int a = 0; a < 3; ++a) dlp[a] = kget(a);
-            Tlp = kget(6);
-        }
-        corrector_pass3<R, NT>(box, dref, uabs, dlp, Tlp, h_dn, h_d1, h_d2, limiter, scr, Phi, Psi);
-        if (recompute) break;
-        R rho1, du[3], T1;
-        const bool ok = pass_frame3<R>(Phi, Psi, Tl, Cv, rho1, du, T1);
-        iters = k + 1;
-        if (!ok) {
-            ++o.fallbacks;
-            last_valid = false;
-            if (!restarted) {
-                restarted = true;
-                R r = R(0), mo[3] = {R(0), R(0), R(0)}, e = R(0);
-#pragma unroll 1
-                for (int s = 0; s < 12; ++s) {
-                    const StagedCell3<R> *c = box.slot(s);
-                    const R rc = c->A[0];
-                    R v2 = R(0);
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        const R d = c->du[face_axis(box.dir, a)] - dref[a];
-                        mo[a] += rc * d;
-                        v2 += d * d;
-                    }
-                    r += rc;
-                    e += rc * (Cv * c->T + R(0.5) * v2);
-                }
-                r /= R(12);
-                e /= R(12);
-                R k2 = R(0);
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    mo[a] /= R(12);
-                    dl[a] = mo[a] / r;
-                    k2 += mo[a] * mo[a];
-                }
-                Tl = (e - R(0.5) * k2 / r) / (Cv * r);
-                continue;
-            }
-            // stop at the last pass that defined a frame
-            done = false;
-            max_iter = 0;
-            continue;
-        }
-        have = true;
-        last_valid = true;
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            kput(a, dl[a]);
-            kput(3 + a, du[a]);
-        }
-        kput(6, Tl);
-        kput(7, T1);
-        kput(8, rho1);
-        if (fixed_iters > 0) {
-            done = iters >= fixed_iters;
-        } else {
-            const R sq = sqrt(Tl);
-            done = fabs(T1 - Tl) <= tol * Tl && fabs(du[0]) <= tol * sq && fabs(du[1]) <= tol * sq && fabs(du[2]) <= tol * sq;
-        }
-#pragma unroll
-        for (int a = 0; a < 3; ++a) dl[a] += du[a];
-        Tl = T1;
-    }
-    o.iters = iters;
-    o.done = done;
-    o.have = have;
-    if (!have) return;
-    R keep_dl[3], out_du[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        keep_dl[a] = kget(a);
-        out_du[a] = kget(3 + a);
-    }
-    const R keep_T = kget(6), out_T = kget(7), out_rho = kget(8);
-    const R invT = R(1) / out_T, rs = sqrt(invT);
-    const R sc = sqrt(keep_T * invT), e = (keep_T - out_T) * invT;
-    Map1<R> X(sc, e, -out_du[0] * rs), Y(sc, e, -out_du[1] * rs), Z(sc, e, -out_du[2] * rs);
-    R Fo[kNF3], Go[kNG3];
-    shift_scale_3d<3, R>(Phi, X, Y, Z, Fo);
-    shift_scale_3d<2, R>(Psi, X, Y, Z, Go);
-    Fo[0] = wb * Fo[0] + we * out_rho;
-#pragma unroll
-    for (int q = 1; q < kNF3; ++q) Fo[q] = wb * Fo[q];
-    Go[0] = wb * Go[0] + we * (Cv - R(1.5)) * out_rho * out_T;
-#pragma unroll
-    for (int q = 1; q < kNG3; ++q) Go[q] = wb * Go[q];
-    from_face<3, R>(Fo, o.F, box.dir);
-    from_face<2, R>(Go, o.G, box.dir);
-    // face axes back to lab axes
-    const R dn = keep_dl[0] + out_du[0], d1 = keep_dl[1] + out_du[1], d2 = keep_dl[2] + out_du[2];
-    const int dir = box.dir;
-    o.du[0] = dir == 0 ? dn : d1;
-    o.du[1] = dir == 1 ? dn : (dir == 0 ? d1 : d2);
-    o.du[2] = dir == 2 ? dn : d2;
-    o.T = out_T;
-}
-
-// Tiles of the 3D face kernel: TX x TY x TZ cells per CTA, one thread per face of each axis
-// (3 TX TY TZ threads), the box [i0-2, i0+TX] x [j0-2, j0+TY] x [k0-2, k0+TZ] staged in
-// dynamic shared memory, followed by the per-thread scratch (the corrector's 3 x 16 values and
-// the 9 kept-frame values); two CTAs per SM.
-template <typename R, int TX_ = 4, int TY_ = 4, int TZ_ = (sizeof(R) == 4 ? 4 : 2), int MINB_ = 2>
-struct Face3Tile {
-    static constexpr int TX = TX_, TY = TY_, TZ = TZ_;
-    static constexpr int THREADS = 3 * TX * TY * TZ;
-    static constexpr int MINB = MINB_;
-    static constexpr int BX = TX + 3, BY = TY + 3, BZ = TZ + 3;
-    static constexpr size_t tile_bytes = sizeof(StagedCell3<R>) * BX * BY * BZ;
-    static constexpr size_t scratch_bytes = sizeof(R) * (kKeep3 + 9) * THREADS;
-    static constexpr size_t smem = tile_bytes + scratch_bytes;
-    static_assert(smem <= 227 * 1024, "the tile and scratch fit one CTA's shared memory");
-};
-
-template <typename R, typename V = Face3Tile<R>>
-__global__ void __launch_bounds__(V::THREADS, V::MINB)
-face3_kernel(const Params3<R> P)
-{
-    using Tl_ = V;
-    constexpr int TX = Tl_::TX, TY = Tl_::TY, TZ = Tl_::TZ, BX = Tl_::BX, BY = Tl_::BY, BZ = Tl_::BZ, NT = Tl_::THREADS;
-    using W = typename FrameWords<R>::word;
-    extern __shared__ __align__(16) unsigned char f3_dyn[];
-    StagedCell3<R> *tile = reinterpret_cast<StagedCell3<R> *>(f3_dyn);
-    R *scr = reinterpret_cast<R *>(f3_dyn + Tl_::tile_bytes) + threadIdx.x;
-    __shared__ W utile[3];
-
-    const Clock &K = *P.clock;
-    // t_end reached (dt = 0): the step is a no-op; tested after the staging loads, so that
-    // this load's latency overlaps theirs
-    const double step_dt = K.dt;
-    const StepC<R> &KC = step_c<R>(K);
-    const long long i0 = (long long)blockIdx.x * TX, j0 = (long long)blockIdx.y * TY, k0 = (long long)blockIdx.z * TZ;
-
-    const int dir = threadIdx.x / (TX * TY * TZ);
-    const int tl = threadIdx.x - dir * TX * TY * TZ;
-    const int tx = tl % TX, ty = (tl / TX) % TY, tz = tl / (TX * TY);
-    const long long fi = i0 + tx, fj = j0 + ty, fk = k0 + tz;
-    const bool active = fi < P.nx + (dir == 0) && fj < P.ny + (dir == 1) && fk < P.nz + (dir == 2);
-    const long long nf = P.nf(dir), f = active ? P.fidx(dir, fi, fj, fk) : 0;
-    // selects: a run-time index into the parameter arrays would copy them to local memory
-    W *Frm = dir == 0 ? P.ffr[0] : (dir == 1 ? P.ffr[1] : P.ffr[2]);
-    // the face's predictor frame, loaded before the staging so that the loads overlap
-    W uref[3], Tpw;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) uref[a] = active ? Frm[a * nf + f] : fr_word(R(0));
-    Tpw = active ? Frm[3 * nf + f] : fr_word(R(1));
-    // the tile's reference velocity: every thread reads it (the same words), so the
-    // staging needs no barrier before it
-    W ut[3];
-    cell_velocity3<R>(P, i0, j0, k0, ut);
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) utile[a] = ut[a];
-    }
-    for (int t = threadIdx.x; t < BX * BY * BZ; t += blockDim.x) {
-        const int bx = t % BX, by = (t / BX) % BY, bz = t / (BX * BY);
-        load_cell3<R>(P, i0 - 2 + bx, j0 - 2 + by, k0 - 2 + bz, KC.cp, KC.ce, ut, tile[t]);
-    }
-    if (!(step_dt > 0.0)) return;   // the same value in every thread
-    __syncthreads();
-
-    unsigned long long my_iters = 0, my_nonconv = 0, my_fallbacks = 0, my_nonphys = 0;
-    if (active) {
-        FaceBox<R> box;
-        box.tile = tile;
-        box.BX = BX;
-        box.BY = BY;
-        box.bx = tx + 2;
-        box.by = ty + 2;
-        box.bz = tz + 2;
-        box.dir = dir;
-        R *Fout = dir == 0 ? P.ff[0] : (dir == 1 ? P.ff[1] : P.ff[2]);
-        R *Gout = dir == 0 ? P.fg[0] : (dir == 1 ? P.fg[1] : P.fg[2]);
-        const R Tp = R(fr_lead(Tpw));
-        // the predictor in face axes (selects: no run-time indexed array)
-        const W un_w = dir == 0 ? uref[0] : (dir == 1 ? uref[1] : uref[2]);
-        const W u1_w = dir == 0 ? uref[1] : uref[0];
-        const W u2_w = dir == 2 ? uref[1] : uref[2];
-        const W tn_w = dir == 0 ? utile[0] : (dir == 1 ? utile[1] : utile[2]);
-        const W t1_w = dir == 0 ? utile[1] : utile[0];
-        const W t2_w = dir == 2 ? utile[1] : utile[2];
-        const R dref[3] = {R(fr_rel(un_w, tn_w)), R(fr_rel(u1_w, t1_w)), R(fr_rel(u2_w, t2_w))};
-        const R uabs[3] = {R(fr_lead(un_w)), R(fr_lead(u1_w)), R(fr_lead(u2_w))};
-        const R h_dn = dir == 0 ? KC.h_dx : (dir == 1 ? KC.h_dy : KC.h_dz);
-        const R h_d1 = dir == 0 ? KC.h_dy : KC.h_dx;
-        const R h_d2 = dir == 2 ? KC.h_dy : KC.h_dz;
-        FaceOut3<R> o;
-        solve_face3<R, NT>(box, dref, uabs, Tp, h_dn, h_d1, h_d2, P.Cv_r, P.tol_r, KC.wb, KC.we, P.limiter, P.max_iter,
-                           P.fixed_iters, scr, o);
-        my_iters = o.iters;
-        my_nonconv = o.done ? 0 : 1;
-        my_fallbacks = o.fallbacks;
-        if (o.have) {
-#pragma unroll
-            for (int q = 0; q < kNF3; ++q) Fout[q * nf + f] = o.F[q];
-#pragma unroll
-            for (int q = 0; q < kNG3; ++q) Gout[q * nf + f] = o.G[q];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) Frm[a * nf + f] = fr_add(uref[a], o.du[a]);
-            Frm[3 * nf + f] = fr_word(o.T);
-        } else {
-            ++my_nonphys;
-            const R nan = R(__longlong_as_double(0x7ff8000000000000ll));
-#pragma unroll
-            for (int q = 0; q < kNF3; ++q) Fout[q * nf + f] = nan;
-#pragma unroll
-            for (int q = 0; q < kNG3; ++q) Gout[q * nf + f] = nan;
-            fr_store(Frm[3 * nf + f], double(nan));
-        }
-    }
-    unsigned long long n_act = active ? 1ull : 0ull;
-    my_iters = warp_sum_count(my_iters);
-    my_nonconv = warp_sum_count(my_nonconv);
-    my_fallbacks = warp_sum_count(my_fallbacks);
-    my_nonphys = warp_sum_count(my_nonphys);
-    n_act = warp_sum_count(n_act);
-    if ((threadIdx.x & 31) == 0 && n_act) {
-        atomicAdd(&P.diag->face_iters, my_iters);
-        atomicAdd(&P.diag->face_solves, n_act);
-        if (my_nonconv) { atomicAdd(&P.diag->nonconv, my_nonconv); atomicOr(&P.diag->flags, FLAG_NOT_CONVERGED); }
-        if (my_fallbacks) atomicAdd(&P.diag->fallbacks, my_fallbacks);
-        if (my_nonphys) { atomicAdd(&P.diag->nonphys, my_nonphys); atomicOr(&P.diag->flags, FLAG_NONPHYSICAL); }
-    }
 }
 
 // ---------------------------------------------------------------- cell update

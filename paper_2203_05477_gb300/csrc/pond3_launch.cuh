@@ -3,16 +3,17 @@
 
 #include <cstdio>
 
-#include "pond3.cuh"
+#include "pond_face3.cuh"
 
 namespace pond {
 
 // dynamic shared memory of the face kernel above the default limit
 template <typename R>
 cudaError_t prepare3();
-// the face kernel of tile variant v (0 .. face3_variant_count - 1) and the cell kernel of
-// block variant v (0 .. cell3_variant_count - 1); names for the autotuner's report
+// the face kernel of tile variant v (0 .. face3_variant_count - 1) with its tail kernel (two
+// launches), and the cell kernel of block variant v (0 .. cell3_variant_count - 1); names for the autotuner's report
 constexpr int face3_variant_count = 3, cell3_variant_count = 3;
+constexpr int launches_per_step3 = 3;
 template <typename R>
 void launch_face3(int v, const Params3<R> &P, cudaStream_t st);
 template <typename R>

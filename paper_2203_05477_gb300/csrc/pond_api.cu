@@ -918,6 +918,7 @@ pond_status setup3(pond_state *s)
         o_ffr[a] = take(sizeof(W) * 4 * nf);
     }
     const size_t o_clock = take(sizeof(pond::Clock)), o_diag = take(sizeof(pond::Diag));
+    const size_t o_tail = take(sizeof(pond::TailList)), o_items = take(sizeof(unsigned long long) * nf_all);
     size_t stage = std::max<size_t>(5 * size_t(n), size_t(pond::kNF3 + pond::kNG3 + 4) * size_t(n));
     stage = std::max<size_t>(stage, 4 * size_t(nf_all));
     stage += 2 * (size_t(kReduceBlocks) * 8 + 8);
@@ -935,6 +936,10 @@ pond_status setup3(pond_state *s)
     }
     P.clock = reinterpret_cast<pond::Clock *>(s->base + o_clock);
     P.diag = reinterpret_cast<pond::Diag *>(s->base + o_diag);
+    P.tail = reinterpret_cast<pond::TailList *>(s->base + o_tail);
+    P.tail_items = reinterpret_cast<unsigned long long *>(s->base + o_items);
+    P.sms = s->sms;
+    P.tail_at = pond::tail3_faces<R>(nf_all, s->sms, s->opts.fixed_iters);
     s->clock = P.clock;
     s->diag = P.diag;
     s->stage = reinterpret_cast<double *>(s->base + o_stage);
@@ -992,13 +997,13 @@ pond_status step3_impl(pond_state *s, int64_t n_steps)
         }
         while (left >= kGraphSteps) {
             CUDA_TRY(cudaGraphLaunch(s->graph_exec, s->stream));
-            s->launches += 2 * kGraphSteps;
+            s->launches += pond::launches_per_step3 * kGraphSteps;
             left -= kGraphSteps;
         }
     }
     for (; left > 0; --left) {
         launch_step3<R>(s);
-        s->launches += 2;
+        s->launches += pond::launches_per_step3;
     }
     CUDA_TRY(cudaGetLastError());
     return POND_OK;
@@ -1017,7 +1022,7 @@ pond_status step3_timed_impl(pond_state *s, int64_t n_steps, double *ms)
         pond::launch_cell3<R>(s->cell_v, P, s->stream);
         CUDA_TRY(cudaEventRecord(ev[2 * k + 2], s->stream));
     }
-    s->launches += 2 * n_steps;
+    s->launches += pond::launches_per_step3 * n_steps;
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaEventSynchronize(ev.back()));
     for (int64_t k = 0; k < n_steps; ++k) {
@@ -2075,7 +2080,7 @@ pond_status time_3d_variant(pond_state *s, const char *saved, int steps, int whi
         pond::launch_cell3<R>(s->cell_v, P, s->stream);
         if (which == 1) CUDA_TRY(cudaEventRecord(ev[2 * k + 1], s->stream));
     }
-    s->launches += int64_t(steps + 1) * 2;
+    s->launches += int64_t(steps + 1) * pond::launches_per_step3;
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaEventSynchronize(ev.back()));
     double sum = 0.0;

@@ -14,15 +14,16 @@ unsigned blocks_of(long long n, int threads) { return unsigned((n + threads - 1)
 }  // namespace
 
 // Tile variants of the 3D face kernel (the autotuner's search space; entry 0 is the default):
-// TX x TY x TZ cells and CTAs per SM for the register budget.
+// TX x TY x TZ cells and CTAs per SM for the register budget.  FP32 tiles are within 1% of one another;
+// FP64 ms (explosion 64^3 / 25 x 23 x 21): 4 x 4 x 2 22.8 / 2.2, 8 x 4 x 2 25.2 / 2.9, 8 x 2 x 2 29.7 / 2.5.
 template <typename R, int V>
 struct Face3Var;
 template <typename R>
-struct Face3Var<R, 0> { using type = Face3Tile<R>; };
+struct Face3Var<R, 0> { using type = std::conditional_t<sizeof(R) == 4, Face3Tile<R, 4, 4, 4, 2>, Face3Tile<R, 4, 4, 2, 2>>; };
 template <typename R>
-struct Face3Var<R, 1> { using type = std::conditional_t<sizeof(R) == 4, Face3Tile<R, 4, 4, 2, 3>, Face3Tile<R, 4, 4, 4, 1>>; };
+struct Face3Var<R, 1> { using type = std::conditional_t<sizeof(R) == 4, Face3Tile<R, 4, 4, 2, 4>, Face3Tile<R, 8, 4, 2, 1>>; };
 template <typename R>
-struct Face3Var<R, 2> { using type = std::conditional_t<sizeof(R) == 4, Face3Tile<R, 8, 4, 2, 2>, Face3Tile<R, 4, 2, 2, 3>>; };
+struct Face3Var<R, 2> { using type = std::conditional_t<sizeof(R) == 4, Face3Tile<R, 8, 4, 2, 2>, Face3Tile<R, 8, 2, 2, 2>>; };
 
 template <typename R, int V>
 cudaError_t prepare3_one()
@@ -46,6 +47,7 @@ void launch_face3_one(const Params3<R> &P, cudaStream_t st)
     using T = typename Face3Var<R, V>::type;
     const dim3 g(unsigned((P.nx + T::TX) / T::TX), unsigned((P.ny + T::TY) / T::TY), unsigned((P.nz + T::TZ) / T::TZ));
     face3_kernel<R, T><<<g, T::THREADS, T::smem, st>>>(P);
+    face3_tail_kernel<R><<<3 * P.sms, kTailThreads3, 0, st>>>(P);
 }
 
 template <typename R>
