@@ -96,8 +96,9 @@ struct pond_state {
     pond_grid3 grid3{};
     alignas(16) unsigned char params3[sizeof(pond::Params3<double>)];
     int64_t launches = 0;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t graph_exec = nullptr;
+    // the captured runs of steps, one for each set of planes the run starts from (sl_parity)
+    cudaGraph_t graph[2] = {nullptr, nullptr};
+    cudaGraphExec_t graph_exec[2] = {nullptr, nullptr};
     // learned face-gauge predictor
     float *mlp = nullptr, *mlp_m = nullptr, *mlp_v = nullptr, *mlp_grad = nullptr, *mlp_loss = nullptr;
     unsigned int *mlp_err = nullptr;
@@ -115,9 +116,9 @@ struct pond_state {
     // tensor maps of the two state buffers for the TMA-staged face variant (D2Q16, FP32)
     pond::StageMaps stage_maps[2] = {};
     // semi-Lagrangian scheme and fused steps: the state alternates between two sets of
-    // planes; sl_parity counts the swaps, graph_parity is the parity a captured graph starts at
+    // planes; sl_parity counts the swaps
     int scheme = POND_FV;
-    int sl_parity = 0, graph_parity = 0;
+    int sl_parity = 0;
     // batched tubes
     bool batch = false;
     int64_t n_tubes = 0, ncell = 0, nface = 0, steps_taken = 0;
@@ -467,25 +468,27 @@ void launch_step(pond_state *s, bool collect = false)
     pond::launch_cell_any<D, R>(s->cell_v, P, s->stream);
 }
 
-// Releases the captured step graph (it is captured again on the next long step).
+// Releases the captured step graphs (captured again on the next long step).
 void drop_graph(pond_state *s)
 {
-    if (s->graph_exec) cudaGraphExecDestroy(s->graph_exec);
-    if (s->graph) cudaGraphDestroy(s->graph);
-    s->graph_exec = nullptr;
-    s->graph = nullptr;
+    for (int p = 0; p < 2; ++p) {
+        if (s->graph_exec[p]) cudaGraphExecDestroy(s->graph_exec[p]);
+        if (s->graph[p]) cudaGraphDestroy(s->graph[p]);
+        s->graph_exec[p] = nullptr;
+        s->graph[p] = nullptr;
+    }
 }
 
 // Instantiates a captured graph and keeps both on the state; on failure neither is kept.
-pond_status keep_graph(pond_state *s, cudaGraph_t g)
+pond_status keep_graph(pond_state *s, cudaGraph_t g, int parity)
 {
-    const cudaError_t e = cudaGraphInstantiate(&s->graph_exec, g, 0);
+    const cudaError_t e = cudaGraphInstantiate(&s->graph_exec[parity], g, 0);
     if (e != cudaSuccess) {
         cudaGraphDestroy(g);
-        s->graph_exec = nullptr;
+        s->graph_exec[parity] = nullptr;
         return fail(POND_ERR_CUDA, "cudaGraphInstantiate: %s", cudaGetErrorString(e));
     }
-    s->graph = g;
+    s->graph[parity] = g;
     return POND_OK;
 }
 
@@ -493,24 +496,21 @@ template <int D, typename R>
 pond_status step_impl(pond_state *s, int64_t n_steps)
 {
     int64_t left = n_steps;
-    if (left >= kGraphSteps && s->graph_exec && s->graph_parity != s->sl_parity) {
-        // the graph was captured starting from the other buffer
-        drop_graph(s);
-    }
     if (left >= kGraphSteps) {
-        if (!s->graph_exec) {
-            s->graph_parity = s->sl_parity;
+        const int parity = s->sl_parity;   // an even number of steps: the same again after each run
+        static_assert(kGraphSteps % 2 == 0, "a run ends on the planes it starts from");
+        if (!s->graph_exec[parity]) {
             CUDA_TRY(cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal));
             const int64_t before = s->launches;
             for (int k = 0; k < kGraphSteps; ++k) launch_step<D, R>(s);
             s->launches = before;
             cudaGraph_t g = nullptr;
             CUDA_TRY(cudaStreamEndCapture(s->stream, &g));
-            if (pond_status st = keep_graph(s, g)) return st;
+            if (pond_status st = keep_graph(s, g, parity)) return st;
         }
         const int per_step = (s->scheme == POND_SL || fused_step<D, R>(s, false)) ? 1 : 2 + ((D == 2 && s->learned) ? 1 : 0);
         while (left >= kGraphSteps) {
-            CUDA_TRY(cudaGraphLaunch(s->graph_exec, s->stream));
+            CUDA_TRY(cudaGraphLaunch(s->graph_exec[parity], s->stream));
             s->launches += per_step * kGraphSteps;
             left -= kGraphSteps;
         }
@@ -988,15 +988,15 @@ pond_status step3_impl(pond_state *s, int64_t n_steps)
 {
     int64_t left = n_steps;
     if (left >= kGraphSteps) {
-        if (!s->graph_exec) {
+        if (!s->graph_exec[0]) {
             CUDA_TRY(cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal));
             for (int k = 0; k < kGraphSteps; ++k) launch_step3<R>(s);
             cudaGraph_t g = nullptr;
             CUDA_TRY(cudaStreamEndCapture(s->stream, &g));
-            if (pond_status st = keep_graph(s, g)) return st;
+            if (pond_status st = keep_graph(s, g, 0)) return st;
         }
         while (left >= kGraphSteps) {
-            CUDA_TRY(cudaGraphLaunch(s->graph_exec, s->stream));
+            CUDA_TRY(cudaGraphLaunch(s->graph_exec[0], s->stream));
             s->launches += pond::launches_per_step3 * kGraphSteps;
             left -= kGraphSteps;
         }
@@ -1204,6 +1204,7 @@ pond_status pond_init(const pond_grid *grid, pond_velset velset, double gamma, d
     }
     if (st == POND_OK) st = reset_clock(s);
     if (st != POND_OK) { pond_destroy(s); return st; }
+    if (D == 1 && s->scheme == POND_FV) s->tube_v = 1 + pond::chunk_default(s->grid.nx, s->sms);
     s->learned = D == 2 && opts->learned != 0;
     if (s->learned) {
         if (s->prec == POND_FP32) params_of<2, float>(s).use_learned = 1;

@@ -18,6 +18,10 @@
 // (u, T) as a float-float pair and the face predictor as plain floats, so its inner loops
 // issue no FP64 instruction: a face frame and the cells it reads are handled as FP32
 // offsets from one reference velocity per chunk.
+//
+// FP64 tubes take the shift-form pass (pass1), which brought 136 tubes of 119 to 238 cells from
+// 343 to 226 us a step (GB300).  The FP32 pass stays node by node: where a corrector cycles
+// without converging its result depends on the rounding, and batches hold such faces.
 #pragma once
 
 #include "pond_kernels.cuh"
@@ -69,16 +73,6 @@ __device__ __forceinline__ void tube_stage(const TubeParams<R> &P, int cur, long
     o.B[2] = cp * P.sg[cur][2 * n + c];
     o.du[0] = R(fr_rel(P.sfr[cur][c], uref));
     o.T = T;
-}
-
-// volatile reads of a parked value (the compiler may not forward the stored registers)
-template <typename R>
-__device__ __forceinline__ R vload(const R *p) { return *reinterpret_cast<const volatile R *>(p); }
-__device__ __forceinline__ double vload_word(const double *p) { return vload(p); }
-__device__ __forceinline__ ffloat vload_word(const ffloat *p)
-{
-    const volatile float *q = reinterpret_cast<const volatile float *>(p);
-    return ffloat{q[0], q[1]};
 }
 
 // per-step constants of one tube (Eqs. FinalUpdateDUGKS, Fbarplus, FluxTransf), formed in
@@ -216,7 +210,7 @@ tube_kernel(const TubeParams<R> P, int steps, int cur0)
                 const R dref[1] = {R(fr_rel(fu_in[f_off + k], utile))};
                 const R uabs[1] = {R(fr_lead(fu_in[f_off + k]))};
                 FaceOut<1, R> o;
-                solve_face<1, R, false, 0, false, sizeof(R) == 4 ? 1 : 0>(cells, false, dref, uabs, R(fT_in[f_off + k]), cfg, o,
+                solve_face<1, R, false, 0, sizeof(R) == 8, sizeof(R) == 4 ? 1 : 0>(cells, false, dref, uabs, R(fT_in[f_off + k]), cfg, o,
                                                                FaceScratch{kept + (sizeof(R) == 4 ? threadIdx.x : 0), THREADS});
                 const bool owned = f < nc || k == L;
                 if (owned) {
@@ -278,11 +272,11 @@ tube_kernel(const TubeParams<R> P, int steps, int cur0)
                 for (int side = 0; side < 2; ++side) {
                     const int f = t + side;
                     const R dv[1] = {faceU[warp][f] - duc};
-                    add_face_flux<1, R>(faceF[warp][f], faceG[warp][f], dv, faceT[warp][f], Tcr, invTc, rsqTc, 0,
+                    add_face_flux<1, R, false, sizeof(R) == 8>(faceF[warp][f], faceG[warp][f], dv, faceT[warp][f], Tcr, invTc, rsqTc, 0,
                                         side ? sx : -sx, sqTc, ucr, H, G);
                 }
                 R Ho[4], Go[3], du[1], dT;
-                bool ok = cell_finish<1, R>(H, G, invTc, sqTc, CvR, Ho, Go, du, dT);
+                bool ok = cell_finish<1, R, sizeof(R) == 8>(H, G, invTc, sqTc, CvR, Ho, Go, du, dT);
                 const CellW un = fr_add(uc, du[0]);
                 const CellW Tn = fr_add(Tc, Tcr * dT);
                 const R unr = R(fr_lead(un)), Tnr = R(fr_lead(Tn));

@@ -33,36 +33,6 @@
 
 namespace pond {
 
-// ------------------------------------------------------------ (f, g) pairs
-
-template <typename R> struct FG;
-template <> struct FG<float> { float2 v; };
-template <> struct FG<double> { double f, g; };
-__device__ __forceinline__ FG<float> fg(float f, float g) { return {make_float2(f, g)}; }
-__device__ __forceinline__ FG<double> fg(double f, double g) { return {f, g}; }
-__device__ __forceinline__ FG<float> operator+(FG<float> a, FG<float> b) { return {__fadd2_rn(a.v, b.v)}; }
-__device__ __forceinline__ FG<double> operator+(FG<double> a, FG<double> b) { return {a.f + b.f, a.g + b.g}; }
-__device__ __forceinline__ FG<float> operator-(FG<float> a, FG<float> b) { return {__fadd2_rn(a.v, make_float2(-b.v.x, -b.v.y))}; }
-__device__ __forceinline__ FG<double> operator-(FG<double> a, FG<double> b) { return {a.f - b.f, a.g - b.g}; }
-__device__ __forceinline__ FG<float> operator*(FG<float> a, float c) { return {__fmul2_rn(a.v, make_float2(c, c))}; }
-__device__ __forceinline__ FG<double> operator*(FG<double> a, double c) { return {a.f * c, a.g * c}; }
-__device__ __forceinline__ FG<float> fgfma(FG<float> a, float c, FG<float> b) { return {__ffma2_rn(a.v, make_float2(c, c), b.v)}; }
-__device__ __forceinline__ FG<double> fgfma(FG<double> a, double c, FG<double> b) { return {fma(a.f, c, b.f), fma(a.g, c, b.g)}; }
-__device__ __forceinline__ float fpart(const FG<float> &a) { return a.v.x; }
-__device__ __forceinline__ float gpart(const FG<float> &a) { return a.v.y; }
-__device__ __forceinline__ double fpart(const FG<double> &a) { return a.f; }
-__device__ __forceinline__ double gpart(const FG<double> &a) { return a.g; }
-// the f part increased by x c
-__device__ __forceinline__ void add_f(FG<float> &a, float x, float c) { a.v.x = fmaf(x, c, a.v.x); }
-__device__ __forceinline__ void add_f(FG<double> &a, double x, double c) { a.f = fma(x, c, a.f); }
-__device__ __forceinline__ FG<float> vanleer_half(FG<float> a, FG<float> b) { return {vanleer_half(Lane2{a.v}, Lane2{b.v}).v}; }
-__device__ __forceinline__ FG<double> vanleer_half(FG<double> a, FG<double> b)
-{
-    return {vanleer_half(a.f, b.f), vanleer_half(a.g, b.g)};
-}
-__device__ __forceinline__ FG<float> vminmod(FG<float> a, FG<float> b) { return {vminmod(Lane2{a.v}, Lane2{b.v}).v}; }
-__device__ __forceinline__ FG<double> vminmod(FG<double> a, FG<double> b) { return {vminmod(a.f, b.f), vminmod(a.g, b.g)}; }
-
 // ------------------------------------------------------------ staged cells
 
 // A staged cell: f 000 and 111, g 000, T, then per lab axis a (others b < c) nine words: f 2a, f 3a,

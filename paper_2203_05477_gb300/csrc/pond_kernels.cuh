@@ -19,6 +19,7 @@
 #include <cuda.h>   // CUtensorMap (the type only; maps are encoded through the runtime's driver entry point)
 
 #include "pond_core.cuh"
+#include "pond_vec.cuh"
 #include "pond_mlp.cuh"
 
 namespace pond {
@@ -91,6 +92,16 @@ __device__ __forceinline__ ffloat fr_add(ffloat x, float d)
 }
 
 
+// volatile reads of a parked value (the compiler may not forward the stored registers)
+template <typename R>
+__device__ __forceinline__ R vload(const R *p) { return *reinterpret_cast<const volatile R *>(p); }
+__device__ __forceinline__ double vload_word(const double *p) { return vload(p); }
+__device__ __forceinline__ ffloat vload_word(const ffloat *p)
+{
+    const volatile float *q = reinterpret_cast<const volatile float *>(p);
+    return ffloat{q[0], q[1]};
+}
+
 enum { BC_TRANSMISSIVE = 0, BC_PERIODIC = 1, BC_INFLOW = 2, BC_REFLECTIVE = 3 };
 enum { FLAG_NONPHYSICAL = 1u, FLAG_NOT_CONVERGED = 2u, FLAG_TIMEOUT = 4u };
 
@@ -122,29 +133,28 @@ __host__ __device__ __forceinline__ const StepC<R> &step_c(const Clock &K)
     else return K.kf;
 }
 
-__host__ __device__ inline void set_step_constants(Clock &c, double dt)
+// The constants of a step of dt, by the first warp of a block: lane k forms the k-th quotient of
+// StepC.  FP64 runs at 1/64 of the FP32 rate, and the fifteen divisions in a row by one thread took
+// 4 us at the end of every step's cell kernel (its whole time is 8 us on a tube of 200 cells).
+__device__ __forceinline__ void step_constants_by_lanes(Clock &c, double dt)
 {
-    const double tau = c.tau, h = 0.5 * dt;
-    c.dt = dt;
-    StepC<double> &k = c.kd;
-    k.ca = (2.0 * tau - dt) / (2.0 * tau + dt);
-    k.cb = 2.0 * dt / (2.0 * tau + dt);
-    k.cp = (2.0 * tau - h) / (2.0 * tau + dt);
-    k.ce = 3.0 * h / (2.0 * tau + dt);
-    k.wb = 2.0 * tau / (2.0 * tau + h);
-    k.we = h / (2.0 * tau + h);
-    k.h_dx = h / c.dx;
-    k.h_dy = h / c.dy;
-    k.dt_dx = dt / c.dx;
-    k.dt_dy = dt / c.dy;
-    k.inv_dx = 1.0 / c.dx;
-    k.inv_dy = 1.0 / c.dy;
-    k.h_dz = h / c.dz;
-    k.dt_dz = dt / c.dz;
-    k.inv_dz = 1.0 / c.dz;
-    c.kf = StepC<float>{float(k.ca),   float(k.cb),   float(k.cp),    float(k.ce),    float(k.wb),     float(k.we),
-                        float(k.h_dx), float(k.h_dy), float(k.dt_dx), float(k.dt_dy), float(k.inv_dx), float(k.inv_dy),
-                        float(k.h_dz), float(k.dt_dz), float(k.inv_dz)};
+    const int k = threadIdx.x & 31;
+    const double tau = c.tau, h = 0.5 * dt, dx = c.dx, dy = c.dy, dz = c.dz;
+    const double num[15] = {2.0 * tau - dt, 2.0 * dt, 2.0 * tau - h, 3.0 * h, 2.0 * tau, h, h, h, dt, dt, 1.0, 1.0, h, dt, 1.0};
+    const double den[15] = {2.0 * tau + dt, 2.0 * tau + dt, 2.0 * tau + dt, 2.0 * tau + dt, 2.0 * tau + h, 2.0 * tau + h,
+                            dx, dy, dx, dy, dx, dy, dz, dz, dz};
+    double a = 1.0, b = 1.0;
+#pragma unroll
+    for (int q = 0; q < 15; ++q) {
+        a = k == q ? num[q] : a;
+        b = k == q ? den[q] : b;
+    }
+    static_assert(sizeof(StepC<double>) == 15 * sizeof(double), "fifteen quotients");
+    if (k < 15) {
+        const double v = a / b;
+        reinterpret_cast<double *>(&c.kd)[k] = v;
+        reinterpret_cast<float *>(&c.kf)[k] = float(v);
+    }
 }
 
 struct Diag {
@@ -637,6 +647,156 @@ __host__ __device__ constexpr int face_scratch_slots(int level) { return level >
 // slots of the last valid pass's frames (kept across the passes, read after the loop)
 __host__ __device__ constexpr int face_keep_slot(int level) { return level > 1 ? 12 : 8; }
 
+// One corrector pass at a D1Q4 face (Grad projection): the four stencil cells in the pass frame
+// (shift form), the outer differences formed in Hermite space, the nodes +-c evaluated as even and
+// odd parts.  A node takes its upwind cell's value and the limited slope of the centre difference
+// and its side's outer one, which enter the limiter symmetrically.  f rides
+// with g in (f, g) pairs for the orders both have (packed FP32x2 in FP32).  About 240 instructions in
+// FP32 against 420 for the node-by-node pass with its maps; 330 FP64 operations against 600.
+// cell(s): the staged cell at slot s (LL, L, R, RR); rel(cell): its velocity less the pass frame's.
+template <typename R, typename CELL, typename REL>
+__device__ __forceinline__ void pass1(CELL &&cell, REL &&rel, R Tl, R un, R h_dn, int limiter, R *Phi, R *Psi)
+{
+    const R invTl = w_rcp<R>(Tl), rsqTl = w_sqrt<R>(invTl), sqTl = Tl * rsqTl;
+    struct Set {
+        FG<R> q[3];   // orders 0..2 of (f, g)
+        R f3;
+    };
+    auto move = [&](int slot) {
+        const auto c = cell(slot);
+        const R s = w_sqrt<R>(c.T * invTl), e = (c.T - Tl) * invTl, d = rel(c) * rsqTl, s2 = e + R(1), s3 = s2 * s;
+        const R F1 = d * c.A[0], q = vfma(s2, c.A[2], e * c.A[0]), F2 = vfma(d, F1, q);   // staged f: zero first order
+        const R b1 = s * c.B[1], G1 = vfma(d, c.B[0], b1), G2 = vfma(d, G1 + b1, vfma(s2, c.B[2], e * c.B[0]));
+        Set o;
+        o.q[0] = fg(c.A[0], c.B[0]);
+        o.q[1] = fg(F1, G1);
+        o.q[2] = fg(F2, G2);
+        o.f3 = vfma(s3, c.A[3], d * vfma(R(2), q, F2));
+        return o;
+    };
+    auto minus = [](const Set &a, const Set &b) {
+        Set o;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) o.q[k] = a.q[k] - b.q[k];
+        o.f3 = a.f3 - b.f3;
+        return o;
+    };
+    const Set L = move(1), Rr = move(2);
+    const Set XL = minus(L, move(0)), XR = minus(move(3), Rr);
+    const R sc = limiter == 1 ? R(1) : R(2);   // the limiter's factor goes into the offset
+    const R k3 = R(0x1.a20bd700c2c3dp-2);      // sqrt(6)/6: He_3(c)/6 = -+ c sqrt(6)/6 at c_lo, c_hi
+    FG<R> S[3];
+    R S3 = R(0);
+#pragma unroll
+    for (int hi = 0; hi < 2; ++hi) {
+        const int np = hi ? 3 : 2, nm = hi ? 0 : 1;   // nodes +c, -c
+        const R c = R(node_c(np)), e2 = R(hen(2, np));
+        auto eval = [&](const Set &a, FG<R> &p, FG<R> &m) {
+            const FG<R> E = fgfma(a.q[2], e2, a.q[0]);
+            FG<R> O = a.q[1];
+            add_f(O, a.f3, hi ? k3 : -k3);
+            p = fgfma(O, c, E);
+            m = fgfma(O, -c, E);
+        };
+        FG<R> lp, lm, rp, rm, ap, am, bp, bm;
+        eval(L, lp, lm);
+        eval(Rr, rp, rm);
+        eval(XL, ap, am);
+        eval(XR, bp, bm);
+        auto value = [&](int n, FG<R> l, FG<R> r, FG<R> a, FG<R> b) {
+            const R vn = vfma(sqTl, R(node_c(n)), un);
+            const bool left = vn > R(0);
+            const R off = sc * ((left ? R(0.5) : R(-0.5)) - vn * h_dn);
+            const FG<R> x = fgsel(left, a, b), u = fgsel(left, l, r), d = r - l;
+            return fgfma(limiter == 1 ? vminmod(x, d) : vanleer_half(x, d), off, u);
+        };
+        const FG<R> vp = value(np, lp, rp, ap, bp), vm = value(nm, lm, rm, am, bm);
+        const FG<R> s = vp + vm, df = vp - vm;
+        const R w0 = R(node_w(np)), w1 = R(node_w(np) * he(1, np)), w2 = R(node_w(np) * he(2, np)), w3 = R(node_w(np) * he(3, np));
+        if (hi == 0) {
+            S[0] = s * w0;
+            S[1] = df * w1;
+            S[2] = s * w2;
+            S3 = fpart(df) * w3;
+        } else {
+            S[0] = fgfma(s, w0, S[0]);
+            S[1] = fgfma(df, w1, S[1]);
+            S[2] = fgfma(s, w2, S[2]);
+            S3 = vfma(fpart(df), w3, S3);
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        Phi[k] = fpart(S[k]);
+        Psi[k] = gpart(S[k]);
+    }
+    Phi[3] = S3;
+}
+
+// The same pass by four lanes per face (j: this lane's place): lane j moves stencil cell j into the frame
+// and evaluates node j, and the moments are summed across the four.  A quarter of the work is
+// serial per lane: 130 FP64 operations a pass against 330 (an FP64 instruction takes 64 cycles
+// whatever the number of lanes), for grids too small to fill the chip with a lane per face.
+template <typename R, typename CELL, typename REL>
+__device__ __forceinline__ void pass1_quad(CELL &&cell, REL &&rel, int j, R Tl, R un, R h_dn, int limiter, R *Phi, R *Psi)
+{
+    const unsigned quad = 0xfu << (threadIdx.x & 28);
+    const int first = threadIdx.x & 28;
+    const R invTl = w_rcp<R>(Tl), rsqTl = w_sqrt<R>(invTl), sqTl = Tl * rsqTl;
+    R F[4], G[3];
+    {
+        const auto c = cell(j);
+        const Move1<R> M(w_sqrt<R>(c.T * invTl), (c.T - Tl) * invTl, rel(c) * rsqTl);
+        const R q = vfma(M.s2, c.A[2], M.e * c.A[0]);
+        F[0] = c.A[0];
+        F[1] = M.d * c.A[0];
+        F[2] = vfma(M.d, F[1], q);
+        F[3] = vfma(M.s3, c.A[3], M.d * vfma(R(2), q, F[2]));
+        M.g(c.B, G);
+    }
+    const NodeTab<R> &tab = node_tab<R>();
+    const R vn = vfma(sqTl, tab.c[j], un);
+    const bool left = vn > R(0);
+    const R h1 = tab.hen[j][1], h2 = tab.hen[j][2], h3 = tab.hen[j][3];
+    // node j of the upwind cell and of the cells below and above it
+    auto eval = [&](int s, R &f, R &g) {
+        const int from = first + s;
+        f = __shfl_sync(quad, F[0], from);
+        g = __shfl_sync(quad, G[0], from);
+        f = vfma(__shfl_sync(quad, F[1], from), h1, f);
+        g = vfma(__shfl_sync(quad, G[1], from), h1, g);
+        f = vfma(__shfl_sync(quad, F[2], from), h2, f);
+        g = vfma(__shfl_sync(quad, G[2], from), h2, g);
+        f = vfma(__shfl_sync(quad, F[3], from), h3, f);
+    };
+    const int u = left ? 1 : 2;
+    R fu, gu, fl, gl, fh, gh;
+    eval(u, fu, gu);
+    eval(u - 1, fl, gl);
+    eval(u + 1, fh, gh);
+    const R off = (left ? R(0.5) : R(-0.5)) - vn * h_dn;
+    if (limiter == 1) {
+        fu = vfma(off, vminmod(fu - fl, fh - fu), fu);
+        gu = vfma(off, vminmod(gu - gl, gh - gu), gu);
+    } else {
+        fu = vfma(R(2) * off, vanleer_half(fu - fl, fh - fu), fu);
+        gu = vfma(R(2) * off, vanleer_half(gu - gl, gh - gu), gu);
+    }
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        R v = tab.whe[j][a] * fu;
+        v += __shfl_xor_sync(quad, v, 1);
+        v += __shfl_xor_sync(quad, v, 2);
+        Phi[a] = v;
+        if (a < 3) {
+            R w = tab.whe[j][a] * gu;
+            w += __shfl_xor_sync(quad, w, 1);
+            w += __shfl_xor_sync(quad, w, 2);
+            Psi[a] = w;
+        }
+    }
+}
+
 // One corrector pass at a face (Sec. III.B.3) in frame (dl, Tl) (velocity relative to the
 // face reference uref): every stencil cell's phi-bar-plus is re-expressed in that frame,
 // limited slopes are formed per population, each population is reconstructed by MUSCL
@@ -654,6 +814,10 @@ __device__ __forceinline__ void corrector_pass(const Stencil<D, R> &cells, const
                                                int limiter, R *Phi, R *Psi, FaceScratch scr = FaceScratch{nullptr, 0})
 {
     static_assert(!SCR || (D == 2 && sizeof(R) == 4 && !EQ), "the scratch variants are FP32 2D Grad passes");
+    if constexpr (D == 1 && OUTER_ONCE && !EQ) {
+        pass1<R>([&](int s) { return fetch<1, R>(cells[s]); },
+                 [&](const StagedCell<1, R> &c) { return c.du[0] - (dref[0] + dl[0]); }, Tl, un_abs, h_dn, limiter, Phi, Psi);
+    } else {
     constexpr int NFC = NCoef<D, 3>::value, NGC = NCoef<D, 2>::value;
     const R invTl = w_rcp<R>(Tl);
     const R rsqTl = w_sqrt<R>(invTl);
@@ -689,8 +853,7 @@ __device__ __forceinline__ void corrector_pass(const Stencil<D, R> &cells, const
     for (int k = 0; k < NGC; ++k) Psi[k] = R(0);
     if constexpr (SCR > 1) scr.store(8, reinterpret_cast<const float *>(Phi), reinterpret_cast<const float *>(Psi));
     // 1D, OUTER_ONCE: the outer neighbours LL and RR in the frame, once per pass (each node
-    // takes the one on its upwind side); else each node transforms its own (fewer live
-    // registers, for kernels that run at a register cap)
+    // takes the one on its upwind side); else each node transforms its own
     R FLL[D == 1 ? NFC : 1], GLL[D == 1 ? NGC : 1], FRR[D == 1 ? NFC : 1], GRR[D == 1 ? NGC : 1];
     if constexpr (D == 1 && OUTER_ONCE) {
 #pragma unroll
@@ -933,6 +1096,7 @@ __device__ __forceinline__ void corrector_pass(const Stencil<D, R> &cells, const
 #pragma unroll 1
         for (int m = 0; m < 4; ++m) node(m);
     }
+    }
 }
 
 // Frame defined by the moments of a pass (Eqs. correctorfieldsrhoDUGKS-TDUGKS), relative
@@ -1000,7 +1164,7 @@ struct FaceOut {
 // KEEP (FP32): 1, the last valid pass's frames wait in two slots of the thread's scratch
 // (after the corrector's own slots) instead of staying live across the next pass; 2, the
 // constants of the face output wait in one more slot
-template <int D, typename R, bool EQ = false, int SCR = 0, bool OUTER_ONCE = true, int KEEP = (SCR > 1 ? 2 : SCR)>
+template <int D, typename R, bool EQ = false, int SCR = 0, bool OUTER_ONCE = true, int KEEP = (SCR > 1 ? 2 : SCR), int LPF = 1>
 __device__ __forceinline__ void solve_face(const Stencil<D, R> &cells, bool swap, const R *dref, const R *uabs,
                                            R Tpred, const FaceCfg<R> &cfg, FaceOut<D, R> &o,
                                            FaceScratch scr = FaceScratch{nullptr, 0})
@@ -1026,9 +1190,17 @@ __device__ __forceinline__ void solve_face(const Stencil<D, R> &cells, bool swap
     bool have = false, done = false, restarted = false, last_valid = false;
     int iters = 0;
     R Phi[NFC], Psi[NGC];
+    auto pass = [&](const R *pdl, R pT) {
+        if constexpr (LPF > 1)
+            pass1_quad<R>([&](int s) { return fetch<1, R>(cells[s]); },
+                          [&](const StagedCell<1, R> &c) { return c.du[0] - (dref[0] + pdl[0]); }, threadIdx.x & (LPF - 1), pT,
+                          uref_n + pdl[0], h_dn, cfg.limiter, Phi, Psi);
+        else
+            corrector_pass<D, R, EQ, SCR, OUTER_ONCE>(cells, dref, pdl, pT, uref_n + pdl[0], D == 2 ? uref_t + pdl[D - 1] : R(0),
+                                                      h_dn, h_dt, cfg.limiter, Phi, Psi, scr);
+    };
     for (int k = 0; k < cfg.max_iter && !done; ++k) {
-        corrector_pass<D, R, EQ, SCR, OUTER_ONCE>(cells, dref, dl, Tl, uref_n + dl[0], D == 2 ? uref_t + dl[D - 1] : R(0),
-                                      h_dn, h_dt, cfg.limiter, Phi, Psi, scr);
+        pass(dl, Tl);
         R rho1, du[D], T1;
         const bool ok = pass_frame<D, R>(Phi, Psi, Tl, Cv, rho1, du, T1);
         iters = k + 1;
@@ -1097,20 +1269,24 @@ __device__ __forceinline__ void solve_face(const Stencil<D, R> &cells, bool swap
     if (have) {
         if (!last_valid) {
             // the last pass defined no frame: recompute the last valid one
-            corrector_pass<D, R, EQ, SCR, OUTER_ONCE>(cells, dref, keep_dl, keep_T, uref_n + keep_dl[0],
-                                          D == 2 ? uref_t + keep_dl[D - 1] : R(0), h_dn, h_dt, cfg.limiter, Phi,
-                                          Psi, scr);
+            pass(keep_dl, keep_T);
         }
         // Eq. (FluxTransf) in the frame of the last valid pass's moments, with the exact
         // co-moving equilibria there: phi = (2 tau phibar + h phi^eq)/(2 tau + h)
         const R invT = w_rcp<R>(out_T);
         const R sk = w_sqrt<R>(keep_T * invT), rsq = w_sqrt<R>(invT);
-        Map1<R> X(sk, (keep_T - out_T) * invT, -out_du[0] * rsq);
-        Map1<R> Y = X;
-        if (D == 2) Y = Map1<R>(sk, (keep_T - out_T) * invT, -out_du[D - 1] * rsq);
         R Fo[NFC], Go[NGC];
-        shift_scale<D, 3, R>(Phi, X, Y, Fo);
-        shift_scale<D, 2, R>(Psi, X, Y, Go);
+        if constexpr (D == 1 && OUTER_ONCE && !EQ) {
+            const Move1<R> M(sk, (keep_T - out_T) * invT, -out_du[0] * rsq);
+            M.f(Phi, Fo);
+            M.g(Psi, Go);
+        } else {
+            Map1<R> X(sk, (keep_T - out_T) * invT, -out_du[0] * rsq);
+            Map1<R> Y = X;
+            if (D == 2) Y = Map1<R>(sk, (keep_T - out_T) * invT, -out_du[D - 1] * rsq);
+            shift_scale<D, 3, R>(Phi, X, Y, Fo);
+            shift_scale<D, 2, R>(Psi, X, Y, Go);
+        }
         R wb = cfg.wb, we = cfg.we, Cvf = Cv;
         if constexpr (KEEP > 1) {
             const float4 w = scr.get(KS + 2);
@@ -1491,12 +1667,29 @@ face_tma_kernel(const Params<D, R> P, const __grid_constant__ StageMaps maps)
 // using c He_r(c) = He_{r+1}(c) + r He_{r-1}(c); He_4 vanishes on the D1Q4 nodes and the
 // Grad forms have no moments above their order, so the product closes on the same orders.
 // invTc, rsqTc: 1/T and 1/sqrt(T) of the cell frame.
-template <int D, typename R, bool EQ = false>
+template <int D, typename R, bool EQ = false, bool SHIFT = D == 1 && !EQ>
 __device__ __forceinline__ void add_face_flux(const R *Fc, const R *Gc, const R *dv, R Tbr, R Tcr, R invTc, R rsqTc,
                                               int axis, R scale, R sqTc, R un, R *H, R *G)
 {
     constexpr int NFC = NCoef<D, 3>::value, NGC = NCoef<D, 2>::value;
     const R s = w_sqrt<R>(Tbr * invTc), e = (Tbr - Tcr) * invTc;
+    if constexpr (SHIFT) {
+        const Move1<R> M(s, e, dv[0] * rsqTc);
+        R F[4], K[3];
+        M.f(Fc, F);
+        M.g(Gc, K);
+        // the flux first, then one addition to the cell's moments: an increment split in two would
+        // round them twice as often
+        const R m = -scale;
+        H[0] = vfma(m, vfma(un, F[0], sqTc * F[1]), H[0]);
+        H[1] = vfma(m, vfma(un, F[1], sqTc * (F[2] + F[0])), H[1]);
+        H[2] = vfma(m, vfma(un, F[2], sqTc * vfma(R(2), F[1], F[3])), H[2]);
+        H[3] = vfma(m, vfma(un, F[3], R(3) * sqTc * F[2]), H[3]);
+        G[0] = vfma(m, vfma(un, K[0], sqTc * K[1]), G[0]);
+        G[1] = vfma(m, vfma(un, K[1], sqTc * (K[2] + K[0])), G[1]);
+        G[2] = vfma(m, vfma(un, K[2], R(2) * sqTc * K[1]), G[2]);
+        return;
+    }
     Map1<R> X(s, e, dv[0] * rsqTc);
     Map1<R> Y = X;
     if constexpr (D == 2) Y = Map1<R>(s, e, dv[1] * rsqTc);
@@ -1616,28 +1809,34 @@ __device__ __forceinline__ void reduce_rate_and_advance(Clock *clock, double rat
     if (threadIdx.x >= 32) return;
     const int nw = (blockDim.x + 31) >> 5;
     b = warp_max_bits(threadIdx.x < nw ? red[threadIdx.x] : 0ull);
-    bool last = false;
+    int last = 0;
     if (threadIdx.x == 0) {
         atomicMax(&clock->rate_bits, b);
         __threadfence();
         const unsigned int nb = gridDim.x * gridDim.y * gridDim.z;
         last = atomicAdd(&clock->blocks_done, 1u) == nb - 1;
     }
-    if (last) {
-        __threadfence();
-        const double rmax = __longlong_as_double((long long)atomicAdd(&clock->rate_bits, 0ull));
-        double t = clock->t;
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    __threadfence();
+    unsigned long long top = 0ull;
+    if (threadIdx.x == 0) top = atomicAdd(&clock->rate_bits, 0ull);
+    const double rmax = __longlong_as_double((long long)__shfl_sync(0xffffffffu, top, 0));
+    double t = clock->t;
+    const double dt_old = clock->dt, t_end = clock->t_end;
+    if (advance) t += dt_old;
+    double dt = clock->cfl / rmax;
+    if (t_end > 0.0) {
+        if (t >= t_end) dt = 0.0;
+        else if (t + dt > t_end) dt = t_end - t;
+    }
+    __syncwarp();   // every lane has read the clock
+    step_constants_by_lanes(*clock, dt);
+    if (threadIdx.x == 0) {
         if (advance) {
-            t += clock->dt;
             clock->t = t;
             clock->steps += 1;
         }
-        double dt = clock->cfl / rmax;
-        if (clock->t_end > 0.0) {
-            if (t >= clock->t_end) dt = 0.0;
-            else if (t + dt > clock->t_end) dt = clock->t_end - t;
-        }
-        set_step_constants(*clock, dt);
+        clock->dt = dt;
         clock->rate_bits = 0ull;
         clock->blocks_done = 0u;
     }
@@ -1648,7 +1847,7 @@ __device__ __forceinline__ void reduce_rate_and_advance(Clock *clock, double rat
 // it (f third order, g second order).  The frame changes by increments formed relative to
 // the old frame, du and dT (T' = T (1 + dT)), which the caller applies to its own
 // representation of the frame.
-template <int D, typename R>
+template <int D, typename R, bool SHIFT = D == 1>
 __device__ __forceinline__ bool cell_finish(const R *H, const R *G, R invTc, R sqTc, R Cv, R *Ho, R *Go, R *du, R &dT)
 {
     const R rsqTc = invTc * sqTc;
@@ -1672,11 +1871,17 @@ __device__ __forceinline__ bool cell_finish(const R *H, const R *G, R invTc, R s
     const R s2 = w_rcp<R>(R(1) + dT);
     const R sc = w_sqrt<R>(s2), e = -dT * s2;
     const R rsqn = rsqTc * sc;
-    Map1<R> X(sc, e, -du[0] * rsqn);
-    Map1<R> Y = X;
-    if constexpr (D == 2) Y = Map1<R>(sc, e, -du[1] * rsqn);
-    shift_scale<D, 3, R>(H, X, Y, Ho);
-    shift_scale<D, 2, R>(G, X, Y, Go);
+    if constexpr (SHIFT) {
+        const Move1<R> M(sc, e, -du[0] * rsqn);
+        M.f(H, Ho);
+        M.g(G, Go);
+    } else {
+        Map1<R> X(sc, e, -du[0] * rsqn);
+        Map1<R> Y = X;
+        if constexpr (D == 2) Y = Map1<R>(sc, e, -du[1] * rsqn);
+        shift_scale<D, 3, R>(H, X, Y, Ho);
+        shift_scale<D, 2, R>(G, X, Y, Go);
+    }
     return ok;
 }
 
@@ -1804,6 +2009,7 @@ struct StepVariant {
     static constexpr int TX = TX_, TY = D == 2 ? TY_ : 1, MINB = MINB_;
     static constexpr int NXF = (TX + 1) * TY, NYF = D == 2 ? TX * (TY + 1) : 0, NF = NXF + NYF;
     static constexpr int THREADS = ((NF + 31) / 32) * 32;
+    static constexpr bool CHUNK = false;
 };
 
 // the faces' populations (coefficients in the face frame, x, y order) and frames in shared
@@ -1917,7 +2123,7 @@ step_kernel(const Params<D, R> P)
             uabs[1] = R(fr_lead(sel(uref, ta)));
         }
         FaceOut<D, R> o;
-        solve_face<D, R, false, 0, sizeof(R) == 4>(cells, swap, dref, uabs, Tp, cfg, o);
+        solve_face<D, R>(cells, swap, dref, uabs, Tp, cfg, o);
         if (owned) {
             my_iters += o.iters;
             my_faces += 1;

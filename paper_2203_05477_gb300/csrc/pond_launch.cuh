@@ -12,6 +12,7 @@
 
 #include "pond_batch.cuh"
 #include "pond_face2.cuh"
+#include "pond_chunk.cuh"
 
 namespace pond {
 
@@ -102,10 +103,19 @@ template <>
 struct StepList<2, double> {
     using type = VList<StepVariant<2, 8, 4, 2>, StepVariant<2, 4, 4, 4>>;
 };
-template <typename R>
-struct StepList<1, R> {
-    using type = VList<StepVariant<1, 124, 1, 4>, StepVariant<1, 60, 1, 8>>;
+template <>
+struct StepList<1, float> {
+    using type = VList<ChunkVariant<1, 4, 4>, ChunkVariant<4, 1, 16>>;
 };
+template <>
+struct StepList<1, double> {
+    using type = VList<ChunkVariant<1, 4, 2>, ChunkVariant<4, 1, 8>>;
+};
+
+// The fused variant of a D1Q4 grid before tuning: four lanes per face while its chunks of 7 cells give
+// each sub-partition at most one warp, else a lane per face (us a step with one / four lanes: tube of
+// 400 cells FP64 104 / 57, 200 cells FP32 13.8 / 12.7, 4 M cells FP32 189 / 549).
+inline int chunk_default(long long nx, int sms) { return nx <= 7ll * 4 * sms ? 1 : 0; }
 
 template <int D, typename R>
 constexpr int step_variants() { return StepList<D, R>::type::size; }
@@ -114,8 +124,10 @@ template <int D, typename R, typename V, typename... Rest>
 void step_name_at(int v, char *buf, size_t n)
 {
     if (v <= 0 || sizeof...(Rest) == 0) {
-        if (D == 2) std::snprintf(buf, n, "step %dx%d cells fused, %d threads, %d CTA/SM", V::TX, V::TY, V::THREADS, V::MINB);
-        else std::snprintf(buf, n, "step %d cells fused, %d threads, %d CTA/SM", V::TX, V::THREADS, V::MINB);
+        if constexpr (V::CHUNK)
+            std::snprintf(buf, n, "step %d cells a warp fused, %d lanes a face, %d threads, %d CTA/SM", V::CELLS, V::LPF, V::THREADS, V::MINB);
+        else
+            std::snprintf(buf, n, "step %dx%d cells fused, %d threads, %d CTA/SM", V::TX, V::TY, V::THREADS, V::MINB);
     } else if constexpr (sizeof...(Rest) > 0) {
         step_name_at<D, R, Rest...>(v - 1, buf, n);
     }

@@ -87,8 +87,15 @@ void launch_cell(int v, const Params<D, R> &P, cudaStream_t st)
 template <int D, typename R, typename V>
 void launch_step_one(const Params<D, R> &P, cudaStream_t st)
 {
-    const dim3 g(unsigned((P.nx + V::TX - 1) / V::TX), D == 2 ? unsigned((P.ny + V::TY - 1) / V::TY) : 1u);
-    step_kernel<D, R, V><<<g, V::THREADS, 0, st>>>(P);
+    if constexpr (V::CHUNK) {
+        // a warp per chunk up to one wave of CTAs, then the warps loop
+        const long long chunks = (P.nx + V::CELLS - 1) / V::CELLS, need = (chunks + V::WARPS - 1) / V::WARPS;
+        const long long wave = (long long)(P.sms > 0 ? P.sms : 1) * V::MINB;
+        chunk_step_kernel<R, V><<<unsigned(need < wave ? need : wave), V::THREADS, 0, st>>>(P);
+    } else {
+        const dim3 g(unsigned((P.nx + V::TX - 1) / V::TX), D == 2 ? unsigned((P.ny + V::TY - 1) / V::TY) : 1u);
+        step_kernel<D, R, V><<<g, V::THREADS, 0, st>>>(P);
+    }
 }
 template <int D, typename R, typename V, typename... Rest>
 void launch_step_at(int v, const Params<D, R> &P, cudaStream_t st)

@@ -98,6 +98,38 @@ __device__ __forceinline__ Lane2 vminmod(Lane2 a, Lane2 b)
 __device__ __forceinline__ double vminmod(double a, double b) { return minmod<double>(a, b); }
 __device__ __forceinline__ float vminmod(float a, float b) { return minmod<float>(a, b); }
 
+// ---- (f, g) pairs: f in lane x and g in lane y of packed FP32x2 instructions in FP32 (worth it where
+// the multiplier is a node constant), two words in FP64
+template <typename R> struct FG;
+template <> struct FG<float> { float2 v; };
+template <> struct FG<double> { double f, g; };
+__device__ __forceinline__ FG<float> fg(float f, float g) { return {make_float2(f, g)}; }
+__device__ __forceinline__ FG<double> fg(double f, double g) { return {f, g}; }
+__device__ __forceinline__ FG<float> operator+(FG<float> a, FG<float> b) { return {__fadd2_rn(a.v, b.v)}; }
+__device__ __forceinline__ FG<double> operator+(FG<double> a, FG<double> b) { return {a.f + b.f, a.g + b.g}; }
+__device__ __forceinline__ FG<float> operator-(FG<float> a, FG<float> b) { return {__fadd2_rn(a.v, make_float2(-b.v.x, -b.v.y))}; }
+__device__ __forceinline__ FG<double> operator-(FG<double> a, FG<double> b) { return {a.f - b.f, a.g - b.g}; }
+__device__ __forceinline__ FG<float> operator*(FG<float> a, float c) { return {__fmul2_rn(a.v, make_float2(c, c))}; }
+__device__ __forceinline__ FG<double> operator*(FG<double> a, double c) { return {a.f * c, a.g * c}; }
+__device__ __forceinline__ FG<float> fgfma(FG<float> a, float c, FG<float> b) { return {__ffma2_rn(a.v, make_float2(c, c), b.v)}; }
+__device__ __forceinline__ FG<double> fgfma(FG<double> a, double c, FG<double> b) { return {fma(a.f, c, b.f), fma(a.g, c, b.g)}; }
+__device__ __forceinline__ float fpart(const FG<float> &a) { return a.v.x; }
+__device__ __forceinline__ float gpart(const FG<float> &a) { return a.v.y; }
+__device__ __forceinline__ double fpart(const FG<double> &a) { return a.f; }
+__device__ __forceinline__ double gpart(const FG<double> &a) { return a.g; }
+// the f part increased by x c
+__device__ __forceinline__ void add_f(FG<float> &a, float x, float c) { a.v.x = fmaf(x, c, a.v.x); }
+__device__ __forceinline__ void add_f(FG<double> &a, double x, double c) { a.f = fma(x, c, a.f); }
+__device__ __forceinline__ FG<float> vanleer_half(FG<float> a, FG<float> b) { return {vanleer_half(Lane2{a.v}, Lane2{b.v}).v}; }
+__device__ __forceinline__ FG<double> vanleer_half(FG<double> a, FG<double> b)
+{
+    return {vanleer_half(a.f, b.f), vanleer_half(a.g, b.g)};
+}
+__device__ __forceinline__ FG<float> vminmod(FG<float> a, FG<float> b) { return {vminmod(Lane2{a.v}, Lane2{b.v}).v}; }
+__device__ __forceinline__ FG<double> vminmod(FG<double> a, FG<double> b) { return {vminmod(a.f, b.f), vminmod(a.g, b.g)}; }
+__device__ __forceinline__ FG<float> fgsel(bool c, FG<float> a, FG<float> b) { return {make_float2(c ? a.v.x : b.v.x, c ? a.v.y : b.v.y)}; }
+__device__ __forceinline__ FG<double> fgsel(bool c, FG<double> a, FG<double> b) { return {c ? a.f : b.f, c ? a.g : b.g}; }
+
 // ---- the regularized change of frame (Sec. II.C) in shift form
 //
 // With s = sqrt(T/T'), e = s^2 - 1 and d = (u - u')/sqrt(T') per axis, the products of the
@@ -109,6 +141,28 @@ __device__ __forceinline__ float vminmod(float a, float b) { return minmod<float
 //     F_21 = dy F_20 + 2 dx a11 + s^3 A_21          (a11 = s^2 A_11)
 // and the same with the axes exchanged: 25 operations in 2D, against 45 for the maps and
 // their products.  The identity (d = e = 0) stays exact.
+template <typename R>
+struct Move1 {
+    R s, e, d, s2, s3;
+    __device__ __forceinline__ Move1(R s_, R e_, R d_) : s(s_), e(e_), d(d_), s2(e_ + R(1)), s3(s2 * s_) {}
+    // orders 0..3 and 0..2, with a first order
+    __device__ __forceinline__ void f(const R *A, R *F) const
+    {
+        const R a1 = s * A[1], q = vfma(s2, A[2], e * A[0]);
+        F[0] = A[0];
+        F[1] = vfma(d, A[0], a1);
+        F[2] = vfma(d, F[1] + a1, q);
+        F[3] = vfma(s3, A[3], vfma(R(3) * e, a1, d * vfma(d, a1, vfma(R(2), q, F[2]))));
+    }
+    __device__ __forceinline__ void g(const R *B, R *G) const
+    {
+        const R b1 = s * B[1];
+        G[0] = B[0];
+        G[1] = vfma(d, B[0], b1);
+        G[2] = vfma(d, G[1] + b1, vfma(s2, B[2], e * B[0]));
+    }
+};
+
 template <typename V>
 struct Move2 {
     V s, e, dx, dy, s2, s3;
