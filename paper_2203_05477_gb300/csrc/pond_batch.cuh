@@ -19,8 +19,11 @@
 // issue no FP64 instruction: a face frame and the cells it reads are handled as FP32
 // offsets from one reference velocity per chunk.
 //
+// Measured (GB300): 4096 tubes of 128 to 4096 cells in FP32 397 us a step (496 before a chunk's
+// loads were issued ahead of the previous chunk's faces, with offsets within a tube in 32 bits and
+// the chunk's state parked in shared memory meanwhile); bound by instruction issue, 1200 a cell.
 // FP64 tubes take the shift-form pass (pass1), which brought 136 tubes of 119 to 238 cells from
-// 343 to 226 us a step (GB300).  The FP32 pass stays node by node: where a corrector cycles
+// 343 to 226 us a step.  The FP32 pass stays node by node: where a corrector cycles
 // without converging its result depends on the rounding, and batches hold such faces.
 #pragma once
 
@@ -56,24 +59,6 @@ struct TubeParams {
     long long *steps_done;        // per tube: steps taken
     Diag *diag;
 };
-
-template <typename R>
-__device__ __forceinline__ void tube_stage(const TubeParams<R> &P, int cur, long long c, R Cvh, R cp, R ce,
-                                           typename FrameWords<R>::word uref, StagedCell<1, R> &o)
-{
-    const long long n = P.ncell;
-    const R rho = P.sf[cur][c];
-    o.A[0] = cp * rho + ce * rho;
-    o.A[1] = R(0);
-    o.A[2] = cp * P.sf[cur][n + c];
-    o.A[3] = cp * P.sf[cur][2 * n + c];
-    const R T = fr_lead(P.sfr[cur][n + c]);
-    o.B[0] = cp * P.sg[cur][c] + ce * Cvh * rho * T;
-    o.B[1] = cp * P.sg[cur][n + c];
-    o.B[2] = cp * P.sg[cur][2 * n + c];
-    o.du[0] = R(fr_rel(P.sfr[cur][c], uref));
-    o.T = T;
-}
 
 // per-step constants of one tube (Eqs. FinalUpdateDUGKS, Fbarplus, FluxTransf), formed in
 // FP64 by one thread and kept in the working precision
@@ -161,56 +146,91 @@ tube_kernel(const TubeParams<R> P, int steps, int cur0)
         cfg.limiter = P.limiter;
         cfg.max_iter = P.max_iter;
         cfg.fixed_iters = P.fixed_iters;
-        const typename TubeParams<R>::FaceW *fu_in = P.fu[cur], *fT_in = P.fT[cur];
-        typename TubeParams<R>::FaceW *fu_out = P.fu[nxt], *fT_out = P.fT[nxt];
+        // offsets within the planes in 32 bits: a batch has fewer than 2^32 cells (each takes over
+        // 100 bytes of device memory)
+        const typename TubeParams<R>::FaceW *fu_in = P.fu[cur] + f_off, *fT_in = P.fT[cur] + f_off;
+        typename TubeParams<R>::FaceW *fu_out = P.fu[nxt] + f_off, *fT_out = P.fT[nxt] + f_off;
         R rate = R(0);
         const long long n = P.ncell;
         const R Cvh = CvR - R(0.5);
+        const R *sf = P.sf[cur] + c_off, *sg = P.sg[cur] + c_off;
+        const CellW *sfr = P.sfr[cur] + c_off;
+        // A chunk's loads are issued before the previous chunk is solved.  Lane l stages cell c0 - 2 + l
+        // (zero-gradient ends) and keeps its state for the update below; lanes 0 and 1 also stage the
+        // right halo c0 + 30, c0 + 31.
+        R rho{}, a2{}, a3{}, b0{}, b1{}, b2{}, fT{};
+        CellW uc{}, Tc{};
+        typename TubeParams<R>::FaceW fu{};
+        R h[6]{}, hT{};
+        CellW hu{};
+        auto load = [&](int chunk) {
+            const int c0 = chunk * kTubeChunk;
+            const unsigned int c = min(max(c0 - 2 + lane, 0), L - 1), k = min(c0 + lane, L);
+            rho = sf[c]; a2 = (sf + n)[c]; a3 = (sf + 2 * n)[c];
+            b0 = sg[c]; b1 = (sg + n)[c]; b2 = (sg + 2 * n)[c];
+            uc = sfr[c]; Tc = (sfr + n)[c];
+            fu = fu_in[k];
+            fT = R(fT_in[k]);
+            if (lane < 2) {
+                const unsigned int q = min(c0 + kTubeChunk + lane, L - 1);
+                h[0] = sf[q]; h[1] = (sf + n)[q]; h[2] = (sf + 2 * n)[q];
+                h[3] = sg[q]; h[4] = (sg + n)[q]; h[5] = (sg + 2 * n)[q];
+                hu = sfr[q];
+                hT = R(fr_lead((sfr + n)[q]));
+            }
+        };
+        auto stage = [&](StagedCell<1, R> &o, R rho, R a2, R a3, R b0, R b1, R b2, CellW u, R T, CellW utile) {
+            o.A[0] = cp * rho + ce * rho;
+            o.A[1] = R(0);
+            o.A[2] = cp * a2;
+            o.A[3] = cp * a3;
+            o.B[0] = cp * b0 + ce * Cvh * rho * T;
+            o.B[1] = cp * b1;
+            o.B[2] = cp * b2;
+            o.du[0] = R(fr_rel(u, utile));
+            o.T = T;
+        };
         // chunks are dealt dynamically: a warp that finishes one takes the next free one, so
         // a warp held up by a chunk whose faces need many corrector passes does fewer chunks
         // (the state and predictors are double-buffered, so the order does not matter)
-        for (int ci = warp; ci * kTubeChunk < L;) {
+        int ci = warp;
+        if (ci * kTubeChunk < L) load(ci);
+        while (ci * kTubeChunk < L) {
             const int c0 = ci * kTubeChunk;
             const int nc = min(kTubeChunk, L - c0);
             // reference velocity of the chunk: its first cell's frame velocity
-            const CellW utile = P.sfr[cur][c_off + c0];
-            // lane l stages cell c0 - 2 + l (zero-gradient ends) and keeps its state for the
-            // update below; lanes 0 and 1 also stage the right halo c0 + 30, c0 + 31
-            const long long c = c_off + min(max(c0 - 2 + lane, 0), L - 1);
-            const R rho = P.sf[cur][c], a2 = P.sf[cur][n + c], a3 = P.sf[cur][2 * n + c];
-            const R b0 = P.sg[cur][c], b1 = P.sg[cur][n + c], b2 = P.sg[cur][2 * n + c];
-            const CellW uc = P.sfr[cur][c], Tc = P.sfr[cur][n + c];
-            const R Tcr = R(fr_lead(Tc));
-            {
-                StagedCell<1, R> &o = wt[lane];
-                o.A[0] = cp * rho + ce * rho;
-                o.A[1] = R(0);
-                o.A[2] = cp * a2;
-                o.A[3] = cp * a3;
-                o.B[0] = cp * b0 + ce * Cvh * rho * Tcr;
-                o.B[1] = cp * b1;
-                o.B[2] = cp * b2;
-                o.du[0] = R(fr_rel(uc, utile));
-                o.T = Tcr;
+            CellW utile;
+            if constexpr (sizeof(R) == 4) {
+                utile.hi = __shfl_sync(0xffffffffu, uc.hi, 2);
+                utile.lo = __shfl_sync(0xffffffffu, uc.lo, 2);
+            } else {
+                utile = __shfl_sync(0xffffffffu, uc, 2);
             }
+            stage(wt[lane], rho, a2, a3, b0, b1, b2, uc, R(fr_lead(Tc)), utile);
+            if (lane < 2) stage(wt[32 + lane], h[0], h[1], h[2], h[3], h[4], h[5], hu, hT, utile);
             raw[warp][0][lane] = rho; raw[warp][1][lane] = a2; raw[warp][2][lane] = a3;
             raw[warp][3][lane] = b0; raw[warp][4][lane] = b1; raw[warp][5][lane] = b2;
             raww[warp][0][lane] = uc; raww[warp][1][lane] = Tc;
-            if (lane < 2) tube_stage<R>(P, cur, c_off + min(c0 + kTubeChunk + lane, L - 1), Cvh, cp, ce, utile, wt[32 + lane]);
+            const typename TubeParams<R>::FaceW fu_c = fu;
+            const R fT_c = fT;
+            int nxt_c = 0;
+            if (lane == 0) nxt_c = atomicAdd(&next_chunk, 1);
+            nxt_c = __shfl_sync(0xffffffffu, nxt_c, 0);
             __syncwarp();
+            if (nxt_c * kTubeChunk < L) load(nxt_c);
             // faces c0 .. c0+nc: face k lies between cells k-1 and k; the last one is also the
             // next chunk's first face, which that chunk owns (except at the tube's end)
             if (lane <= nc) {
                 const int f = lane;
-                const long long k = c0 + f;
+                const int k = c0 + f;
                 Stencil<1, R> cells;   // LL, L, R, RR at wt[f .. f+3]
                 cells.base = &wt[f + 2];
                 cells.sn = 1;
                 cells.st = 0;
-                const R dref[1] = {R(fr_rel(fu_in[f_off + k], utile))};
-                const R uabs[1] = {R(fr_lead(fu_in[f_off + k]))};
+                const R dref[1] = {R(fr_rel(fu_c, utile))};
+                const R uabs[1] = {R(fr_lead(fu_c))};
                 FaceOut<1, R> o;
-                solve_face<1, R, false, 0, sizeof(R) == 8, sizeof(R) == 4 ? 1 : 0>(cells, false, dref, uabs, R(fT_in[f_off + k]), cfg, o,
+                solve_face<1, R, false, 0, sizeof(R) == 8, sizeof(R) == 4 ? 1 : 0>(cells, false, dref, uabs, fT_c, cfg, o,
                                                                FaceScratch{kept + (sizeof(R) == 4 ? threadIdx.x : 0), THREADS});
                 const bool owned = f < nc || k == L;
                 if (owned) {
@@ -228,8 +248,8 @@ tube_kernel(const TubeParams<R> P, int steps, int cur0)
                     faceU[warp][f] = fdu;
                     faceT[warp][f] = o.T;
                     if (owned) {
-                        fu_out[f_off + k] = fr_face(utile, fdu);
-                        fT_out[f_off + k] = o.T;
+                        fu_out[k] = fr_face(utile, fdu);
+                        fT_out[k] = o.T;
                     }
                 } else {
                     if (owned) ++my_nonphys;
@@ -242,8 +262,8 @@ tube_kernel(const TubeParams<R> P, int steps, int cur0)
                     faceU[warp][f] = dref[0];
                     faceT[warp][f] = nan;
                     if (owned) {
-                        fu_out[f_off + k] = fu_in[f_off + k];
-                        fT_out[f_off + k] = nan;
+                        fu_out[k] = fu_c;
+                        fT_out[k] = nan;
                     }
                 }
             }
@@ -255,7 +275,7 @@ tube_kernel(const TubeParams<R> P, int steps, int cur0)
                 const R b0 = vload(&raw[warp][3][lane]), b1 = vload(&raw[warp][4][lane]), b2 = vload(&raw[warp][5][lane]);
                 const CellW uc = vload_word(&raww[warp][0][lane]), Tc = vload_word(&raww[warp][1][lane]);
                 const R Tcr = R(fr_lead(Tc));
-                const long long c = c_off + min(max(c0 - 2 + lane, 0), L - 1);
+                const unsigned int c = c0 + t;   // the cell this lane staged
                 const R duc = wt[lane].du[0];
                 const R invTc = w_rcp<R>(Tcr), rsqTc = w_sqrt<R>(invTc), sqTc = Tcr * rsqTc;
                 R H[4], G[3];
@@ -284,25 +304,25 @@ tube_kernel(const TubeParams<R> P, int steps, int cur0)
                 if (!ok) {
                     ++my_nonphys;
                     tube_bad = 1;
-                    atomicCAS((unsigned long long *)&P.diag->first_bad, (unsigned long long)-1ll, (unsigned long long)c);
+                    atomicCAS((unsigned long long *)&P.diag->first_bad, (unsigned long long)-1ll, (unsigned long long)(c_off + c));
                 }
-                P.sf[nxt][c] = Ho[0];
-                P.sf[nxt][n + c] = Ho[2];
-                P.sf[nxt][2 * n + c] = Ho[3];
-                P.sg[nxt][c] = Go[0];
-                P.sg[nxt][n + c] = Go[1];
-                P.sg[nxt][2 * n + c] = Go[2];
-                P.sfr[nxt][c] = un;
-                P.sfr[nxt][n + c] = Tn;
+                R *osf = P.sf[nxt] + c_off, *osg = P.sg[nxt] + c_off;
+                CellW *osfr = P.sfr[nxt] + c_off;
+                osf[c] = Ho[0];
+                (osf + n)[c] = Ho[2];
+                (osf + 2 * n)[c] = Ho[3];
+                osg[c] = Go[0];
+                (osg + n)[c] = Go[1];
+                (osg + 2 * n)[c] = Go[2];
+                osfr[c] = un;
+                (osfr + n)[c] = Tn;
                 if (ok) {
                     if constexpr (sizeof(R) == 8) rate = fmax(rate, (fabs(unr) + sqrt(Tnr) * kCHi) / dx);
                     else rate = fmaxf(rate, (fabsf(unr) + sqrtf(Tnr) * float(kCHi)) * ks.inv_dx);
                 }
             }
             __syncwarp();   // the chunk's shared records are read before the next chunk restages them
-            int nxt_c = 0;
-            if (lane == 0) nxt_c = atomicAdd(&next_chunk, 1);
-            ci = __shfl_sync(0xffffffffu, nxt_c, 0);
+            ci = nxt_c;
         }
         // the tube's next time step from its CFL maximum (Sec. IV)
         R r = rate;
