@@ -398,13 +398,10 @@ pond_status mlp_setup(pond_state *s)
 // captured graph holds both orders alternately)
 constexpr int kSlThreads = 128;
 
-// D2Q16: tiles of 8 x 8 nodes (FP32) or 8 x 4 (FP64), the per-thread scratch of 140
-// collapsed coefficients in dynamic shared memory
+// D2Q16: tiles of 8 x 8 nodes (FP32) or 8 x 2 (FP64), four threads a node; the nodes' scratch in
+// dynamic shared memory (two CTAs per SM, three in FP64)
 template <typename R>
-struct Sl2Tile {
-    static constexpr int TX = 8, TY = sizeof(R) == 4 ? 8 : 4;
-    static constexpr size_t scratch = size_t(TX) * TY * 140 * sizeof(R);
-};
+using Sl2 = pond::Sl2Tile<R, 8, sizeof(R) == 4 ? 8 : 2, sizeof(R) == 4 ? 2 : 3>;
 
 template <int D, typename R>
 void launch_sl(pond_state *s, pond::Params<D, R> &P)
@@ -412,9 +409,9 @@ void launch_sl(pond_state *s, pond::Params<D, R> &P)
     if constexpr (D == 1) {
         pond::sl_kernel<R, kSlThreads><<<blocks_for(P.nx, kSlThreads), kSlThreads, 0, s->stream>>>(P);
     } else {
-        using T = Sl2Tile<R>;
+        using T = Sl2<R>;
         const dim3 g(unsigned((P.nx + T::TX - 1) / T::TX), unsigned((P.ny + T::TY - 1) / T::TY));
-        pond::sl2_kernel<R, T::TX, T::TY><<<g, T::TX * T::TY, T::scratch, s->stream>>>(P);
+        pond::sl2_kernel<R, T><<<g, T::THREADS, T::scratch, s->stream>>>(P);
     }
     std::swap(P.sf, P.xf);
     std::swap(P.sg, P.xg);
@@ -1184,10 +1181,10 @@ pond_status pond_init(const pond_grid *grid, pond_velset velset, double gamma, d
     if (st == POND_OK && D == 2 && s->scheme == POND_SL) {
         // the 2D semi-Lagrangian kernel's scratch can exceed the default dynamic shared memory
         const cudaError_t ea = s->prec == POND_FP32
-            ? cudaFuncSetAttribute(pond::sl2_kernel<float, Sl2Tile<float>::TX, Sl2Tile<float>::TY>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(Sl2Tile<float>::scratch))
-            : cudaFuncSetAttribute(pond::sl2_kernel<double, Sl2Tile<double>::TX, Sl2Tile<double>::TY>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(Sl2Tile<double>::scratch));
+            ? cudaFuncSetAttribute(pond::sl2_kernel<float, Sl2<float>>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(Sl2<float>::scratch))
+            : cudaFuncSetAttribute(pond::sl2_kernel<double, Sl2<double>>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(Sl2<double>::scratch));
         if (ea != cudaSuccess) st = fail(POND_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(ea));
     }
     if (st == POND_OK && D == 2) {
