@@ -281,8 +281,8 @@ pond_status pond_mlp_gradient(const float *params, const float *x, int ldx, cons
  * framework's caching allocator has reserved the whole device, code that must not add the
  * device-wide synchronization cudaMalloc/cudaFree imply, or code on a path where a failed
  * allocation cannot be handled.  Inputs and outputs are as for pond_mlp_gradient (device
- * arrays owned by the caller).  The activation scratch lives in a fixed device array of
- * the library sized for POND_MLP_NOALLOC_MAX_ROWS rows (about 6.6 MB, held by every GPU that
+ * arrays owned by the caller).  The partial gradients live in a fixed device array of
+ * the library sized for POND_MLP_NOALLOC_MAX_ROWS rows (about 2.1 MB, held by every GPU that
  * loads the library until the process exits); n above that limit returns
  * POND_ERR_INVALID_ARG.  Every call looks up that array's device address in the current
  * context (no allocation); the first call on a device also sets the kernels' shared-memory
@@ -290,8 +290,7 @@ pond_status pond_mlp_gradient(const float *params, const float *x, int ldx, cons
  * stream capture.  All calls share the one array: calls whose work overlaps on the GPU
  * (different streams, or threads calling concurrently) race on it; serialize them.  The
  * call clears *loss and its error word itself, enqueues on `stream`, and waits for it.
- * On POND_ERR_TIMEOUT grad is left as it was (the weight-gradient kernel does not run on
- * incomplete activations) and *loss is undefined. */
+ * On POND_ERR_TIMEOUT grad is left as it was (the partial gradients are not summed) and *loss is undefined. */
 #define POND_MLP_NOALLOC_MAX_ROWS 8192
 pond_status pond_mlp_gradient_noalloc(const float *params, const float *x, int ldx, const float *y, int ldy, int64_t n,
                                       float *grad, float *loss, void *stream);

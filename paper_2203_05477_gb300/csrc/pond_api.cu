@@ -384,7 +384,7 @@ pond_status mlp_setup(pond_state *s)
     mlp_default_params(p);
     CUDA_TRY(cudaMemcpyAsync(s->mlp, p.data(), 4 * M::kParams, cudaMemcpyHostToDevice, s->stream));
     CUDA_TRY(cudaStreamSynchronize(s->stream));
-    CUDA_TRY(cudaFuncSetAttribute(pond::mlp::tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, M::kTileSmem));
+    CUDA_TRY(cudaFuncSetAttribute(M::forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, M::kTileSmem));
     CUDA_TRY(cudaFuncSetAttribute(pond::gauge_predict_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, M::kInferSmem));
     CUDA_TRY(cudaFuncSetAttribute(pond::gauge_predict_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, M::kInferSmem));
     int sms = 0;
@@ -1501,48 +1501,69 @@ pond_status gauge_collect_impl(pond_state *s, int64_t n_steps, float *pairs, int
     return POND_OK;
 }
 
-// scratch of a training minibatch of `rows` rows: the activations out, H1, H2, dOut, dZ1,
-// dZ2, and the partial weight gradients of the split batch
-constexpr size_t kWgradPartBytes = size_t(pond::mlp::kWgradMaxSplit) * pond::mlp::kParams * 4;
-struct TrainScratch {
-    float *out;
-    __nv_bfloat16 *H1, *H2, *dOut, *dZ1, *dZ2;
-    float *part;
-    static constexpr size_t bytes(int64_t rows)
-    {
-        return size_t(rows) * (16 * 4 + 2 * (64 + 64 + 16 + 64 + 64)) + 1024 + kWgradPartBytes + 256;
-    }
-    static TrainScratch carve(char *base, int64_t rows)
-    {
-        TrainScratch t;
-        size_t off = 0;
-        auto take = [&](size_t b) { size_t o = off; off = align_up(off + b, 256); return base + o; };
-        t.part = reinterpret_cast<float *>(take(kWgradPartBytes));
-        t.out = reinterpret_cast<float *>(take(size_t(rows) * 64));
-        t.H1 = reinterpret_cast<__nv_bfloat16 *>(take(size_t(rows) * 128));
-        t.H2 = reinterpret_cast<__nv_bfloat16 *>(take(size_t(rows) * 128));
-        t.dOut = reinterpret_cast<__nv_bfloat16 *>(take(size_t(rows) * 32));
-        t.dZ1 = reinterpret_cast<__nv_bfloat16 *>(take(size_t(rows) * 128));
-        t.dZ2 = reinterpret_cast<__nv_bfloat16 *>(take(size_t(rows) * 128));
-        return t;
-    }
-};
+// partial gradients of a batch of `rows` rows, one for each CTA that takes part
+constexpr int64_t grad_parts(int64_t rows)
+{
+    const int64_t tiles = (rows + pond::mlp::kRows - 1) / pond::mlp::kRows;
+    return tiles < pond::mlp::kGradMaxCtas ? tiles : pond::mlp::kGradMaxCtas;
+}
+constexpr size_t grad_bytes(int64_t rows) { return size_t(grad_parts(rows)) * pond::mlp::kPartStride * sizeof(float); }
 
-// one gradient evaluation: forward, loss, backward through the activations, weight grads
-pond_status mlp_grad_launch(const float *prm, const float *x, int ldx, const float *y, int ldy, int64_t n,
-                            const TrainScratch &t, float *grad, float *loss, unsigned int *err, cudaStream_t st)
+pond_status grad_setup()
+{
+    CUDA_TRY(cudaFuncSetAttribute(pond::mlp::grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, pond::mlp::kGradSmem));
+    return POND_OK;
+}
+
+// one gradient evaluation: forward, loss, backward through the activations, weight grads; part holds
+// grad_bytes(n)
+pond_status mlp_grad_launch(const float *prm, const float *x, int ldx, const float *y, int ldy, int64_t n, float *part,
+                            float *grad, float *loss, unsigned int *err, cudaStream_t st)
 {
     namespace M = pond::mlp;
-    const unsigned tiles = unsigned((n + M::kRows - 1) / M::kRows);
-    M::tile_kernel<<<tiles, M::kThreads, M::kTileSmem, st>>>(prm, x, ldx, y, ldy, n, t.out, t.H1, t.H2, t.dOut, t.dZ1,
-                                                               t.dZ2, loss, err);
-    const int nsplit = M::wgrad_splits(n);
-    M::wgrad_kernel<<<dim3(3, unsigned(nsplit)), M::kThreads, 0, st>>>(x, ldx, t.H1, t.H2, t.dOut, t.dZ1, t.dZ2, n, t.part,
-                                                                          err);
-    M::wgrad_reduce_kernel<<<(M::kParams + 255) / 256, 256, 0, st>>>(t.part, nsplit, grad, err);
+    const int64_t tiles = (n + M::kRows - 1) / M::kRows, per = (tiles + M::kGradMaxCtas - 1) / M::kGradMaxCtas;
+    const unsigned ctas = unsigned((tiles + per - 1) / per);
+    M::grad_kernel<<<ctas, M::kGradThreads, M::kGradSmem, st>>>(prm, x, ldx, y, ldy, n, int(per), part, err);
+    M::grad_reduce_kernel<<<M::kParams / 32 + 1, 256, 0, st>>>(part, int(ctas), grad, loss, err);
     CUDA_TRY(cudaGetLastError());
     return POND_OK;
 }
+
+// Scratch of pond_mlp_gradient: a call holds one slot from its start until its work has run, so
+// calls from several threads and on several streams never share one.  (A cudaMalloc and cudaFree
+// on each call took about 250 us, three times the kernels at 65536 rows.)
+constexpr int kMaxDevices = 64;
+constexpr int kGradSlots = 2;
+constexpr size_t kGradSlotBytes = align_up(size_t(pond::mlp::kGradMaxCtas) * pond::mlp::kPartStride * sizeof(float), 256) + 256;
+static __device__ __align__(256) unsigned char g_grad_scratch[kGradSlots][kGradSlotBytes];
+std::mutex g_grad_mutex;
+bool g_grad_busy[kMaxDevices][kGradSlots] = {};
+
+struct GradSlot {
+    char *base = nullptr;   // null: no slot was free
+    int dev = -1, k = -1;
+    pond_status take()
+    {
+        void *p = nullptr;
+        CUDA_TRY(cudaGetDevice(&dev));
+        if (dev < 0 || dev >= kMaxDevices) return POND_OK;
+        CUDA_TRY(cudaGetSymbolAddress(&p, g_grad_scratch));
+        std::lock_guard<std::mutex> lock(g_grad_mutex);
+        for (int i = 0; i < kGradSlots && k < 0; ++i)
+            if (!g_grad_busy[dev][i]) {
+                g_grad_busy[dev][i] = true;
+                k = i;
+                base = static_cast<char *>(p) + size_t(i) * kGradSlotBytes;
+            }
+        return POND_OK;
+    }
+    ~GradSlot()
+    {
+        if (k < 0) return;
+        std::lock_guard<std::mutex> lock(g_grad_mutex);
+        g_grad_busy[dev][k] = false;
+    }
+};
 
 __device__ unsigned int g_standalone_err;
 __device__ unsigned int g_wait_check_err;
@@ -1577,12 +1598,13 @@ pond_status pond_gauge_train(pond_state *s, const float *pairs, int64_t n, int e
     if (!pairs || n <= 0 || epochs < 1 || batch < 1 || !(lr > 0.f)) return fail(POND_ERR_INVALID_ARG, "bad train arguments");
     if (s->train_rows < batch) {
         dev_free(s, s->train_scratch);
-        s->train_scratch = static_cast<char *>(dev_alloc(s, TrainScratch::bytes(batch)));
+        s->train_rows = 0;
+        s->train_scratch = static_cast<char *>(dev_alloc(s, grad_bytes(batch)));
         if (!s->train_scratch) return fail(POND_ERR_OOM, "training scratch allocation failed");
         s->train_rows = batch;
     }
-    CUDA_TRY(cudaFuncSetAttribute(M::tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, M::kTileSmem));
-    const TrainScratch t = TrainScratch::carve(s->train_scratch, batch);
+    if (pond_status st = grad_setup()) return st;
+    float *part = reinterpret_cast<float *>(s->train_scratch);
     CUDA_TRY(cudaMemsetAsync(s->mlp_err, 0, sizeof(unsigned int), s->stream));
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     for (int ep = 0; ep < epochs; ++ep) {
@@ -1591,14 +1613,14 @@ pond_status pond_gauge_train(pond_state *s, const float *pairs, int64_t n, int e
         for (int64_t b0 = 0; b0 < n; b0 += batch, ++nb) {
             const int64_t rows = std::min<int64_t>(batch, n - b0);
             const float *xb = pairs + b0 * M::kPairStride;
-            pond_status st = mlp_grad_launch(s->mlp, xb, M::kPairStride, xb, M::kPairStride, rows, t, s->mlp_grad,
+            pond_status st = mlp_grad_launch(s->mlp, xb, M::kPairStride, xb, M::kPairStride, rows, part, s->mlp_grad,
                                              s->mlp_loss, s->mlp_err, s->stream);
             if (st != POND_OK) return st;
             ++s->adam_t;
             const float bc1 = 1.f - std::pow(b1, float(s->adam_t)), bc2 = 1.f - std::pow(b2, float(s->adam_t));
             M::adam_kernel<<<(M::kParams + 255) / 256, 256, 0, s->stream>>>(s->mlp, s->mlp_grad, s->mlp_m, s->mlp_v, lr, b1,
                                                                              b2, eps, bc1, bc2);
-            s->launches += 4;   // tile, weight-gradient, reduction and Adam kernels
+            s->launches += 3;   // gradient, reduction and Adam kernels
         }
         CUDA_TRY(cudaGetLastError());
         float l = 0.f;
@@ -1734,12 +1756,11 @@ pond_status pond_mlp_forward(const float *params, const float *x, int ldx, int64
     namespace M = pond::mlp;
     if (!params || !x || !out || n <= 0 || ldx < M::kIn) return fail(POND_ERR_INVALID_ARG, "bad forward arguments");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    CUDA_TRY(cudaFuncSetAttribute(M::tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, M::kTileSmem));
+    CUDA_TRY(cudaFuncSetAttribute(M::forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, M::kTileSmem));
     unsigned int *err = nullptr;
     CUDA_TRY(cudaGetSymbolAddress(reinterpret_cast<void **>(&err), g_standalone_err));
     CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(unsigned int), st));
-    M::tile_kernel<<<unsigned((n + M::kRows - 1) / M::kRows), M::kThreads, M::kTileSmem, st>>>(
-        params, x, ldx, nullptr, 0, n, out, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, err);
+    M::forward_kernel<<<unsigned((n + M::kRows - 1) / M::kRows), M::kThreads, M::kTileSmem, st>>>(params, x, ldx, n, out, err);
     CUDA_TRY(cudaGetLastError());
     unsigned int e = 0;
     CUDA_TRY(cudaMemcpyAsync(&e, err, sizeof(e), cudaMemcpyDeviceToHost, st));
@@ -1755,16 +1776,22 @@ pond_status pond_mlp_gradient(const float *params, const float *x, int ldx, cons
     if (!params || !x || !y || !grad || !loss || n <= 0 || ldx < M::kIn || ldy < M::kIn + M::kOut)
         return fail(POND_ERR_INVALID_ARG, "bad gradient arguments");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    CUDA_TRY(cudaFuncSetAttribute(M::tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, M::kTileSmem));
-    char *scratch = nullptr;
-    CUDA_TRY(cudaMalloc(&scratch, TrainScratch::bytes(n)));
-    unsigned int *err = nullptr;
+    if (pond_status r = grad_setup()) return r;
+    // a slot of the fixed scratch for the length of the call (which waits for its work), or, when
+    // other threads hold them all, an allocation
+    GradSlot slot;
+    if (pond_status r = slot.take()) return r;
+    char *own = nullptr, *scratch = slot.base;
+    if (!scratch) {
+        CUDA_TRY(cudaMalloc(&own, kGradSlotBytes));
+        scratch = own;
+    }
+    unsigned int *err = reinterpret_cast<unsigned int *>(scratch + kGradSlotBytes - 256);
     pond_status r = POND_OK;
-    cudaError_t ce = cudaGetSymbolAddress(reinterpret_cast<void **>(&err), g_standalone_err);
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(err, 0, sizeof(unsigned int), st);
+    cudaError_t ce = cudaMemsetAsync(err, 0, sizeof(unsigned int), st);
     if (ce == cudaSuccess) ce = cudaMemsetAsync(loss, 0, sizeof(float), st);
     if (ce != cudaSuccess) r = fail(POND_ERR_CUDA, "%s", cudaGetErrorString(ce));
-    if (r == POND_OK) r = mlp_grad_launch(params, x, ldx, y, ldy, n, TrainScratch::carve(scratch, n), grad, loss, err, st);
+    if (r == POND_OK) r = mlp_grad_launch(params, x, ldx, y, ldy, n, reinterpret_cast<float *>(scratch), grad, loss, err, st);
     unsigned int e = 0;
     if (r == POND_OK) {
         ce = cudaMemcpyAsync(&e, err, sizeof(e), cudaMemcpyDeviceToHost, st);
@@ -1772,8 +1799,8 @@ pond_status pond_mlp_gradient(const float *params, const float *x, int ldx, cons
         if (ce != cudaSuccess) r = fail(POND_ERR_CUDA, "%s", cudaGetErrorString(ce));
         else if (e) r = fail(POND_ERR_TIMEOUT, "a tensor-core wait timed out");
     }
-    cudaStreamSynchronize(st);
-    cudaFree(scratch);
+    if (r != POND_OK) cudaStreamSynchronize(st);
+    if (own) cudaFree(own);
     return r;
 }
 
@@ -1783,19 +1810,18 @@ pond_status pond_mlp_gradient(const float *params, const float *x, int ldx, cons
 
 namespace {
 
-// Scratch of pond_mlp_gradient_noalloc: the activations of up to POND_MLP_NOALLOC_MAX_ROWS
+// Scratch of pond_mlp_gradient_noalloc: the partial gradients of up to POND_MLP_NOALLOC_MAX_ROWS
 // rows, followed by the error word.  In host code this name only stands for the symbol;
 // its device address comes from cudaGetSymbolAddress for the current device.
-constexpr size_t kNoallocScratch = align_up(TrainScratch::bytes(POND_MLP_NOALLOC_MAX_ROWS), 256) + 256;
+constexpr size_t kNoallocScratch = align_up(grad_bytes(POND_MLP_NOALLOC_MAX_ROWS), 256) + 256;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratch];
 
-constexpr int kMaxDevices = 64;
 std::mutex g_noalloc_mutex;
 bool g_noalloc_ready[kMaxDevices] = {};
 
 // With the caller's device current: the array's device address in the current context
 // (looked up on every call, which allocates nothing, so a context created after a device
-// reset gets its own address) and, once per device, the tile kernel's shared-memory limit.
+// reset gets its own address) and, once per device, the gradient kernel's shared-memory limit.
 pond_status noalloc_setup(unsigned char **out)
 {
     int dev = 0;
@@ -1805,7 +1831,7 @@ pond_status noalloc_setup(unsigned char **out)
     CUDA_TRY(cudaGetSymbolAddress(&p, g_noalloc_scratch));
     std::lock_guard<std::mutex> lock(g_noalloc_mutex);
     if (!g_noalloc_ready[dev]) {
-        CUDA_TRY(cudaFuncSetAttribute(pond::mlp::tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, pond::mlp::kTileSmem));
+        if (pond_status st = grad_setup()) return st;
         g_noalloc_ready[dev] = true;
     }
     *out = static_cast<unsigned char *>(p);
@@ -1828,12 +1854,11 @@ pond_status pond_mlp_gradient_noalloc(const float *params, const float *x, int l
     unsigned char *base = nullptr;
     if (pond_status st = noalloc_setup(&base)) return st;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const TrainScratch t = TrainScratch::carve(reinterpret_cast<char *>(base), POND_MLP_NOALLOC_MAX_ROWS);
     unsigned int *err = reinterpret_cast<unsigned int *>(base + kNoallocScratch - 256);
     // the loss accumulates and the error word is or-ed into: both start at zero
     CUDA_TRY(cudaMemsetAsync(err, 0, sizeof(unsigned int), st));
     CUDA_TRY(cudaMemsetAsync(loss, 0, sizeof(float), st));
-    pond_status r = mlp_grad_launch(params, x, ldx, y, ldy, n, t, grad, loss, err, st);
+    pond_status r = mlp_grad_launch(params, x, ldx, y, ldy, n, reinterpret_cast<float *>(base), grad, loss, err, st);
     if (r != POND_OK) return r;
     unsigned int e = 0;
     CUDA_TRY(cudaMemcpyAsync(&e, err, sizeof(e), cudaMemcpyDeviceToHost, st));

@@ -30,18 +30,14 @@ constexpr int kThreads = 128;      // one thread per row
 constexpr long long kPolls = 1ll << 22;   // bound on every mbarrier wait
 constexpr int kPairStride = 52;    // features (48), targets (3), corrector passes of the face
 
-// shared-memory plan of the tile kernel (byte offsets, 128-aligned)
+// shared-memory plan of the forward kernel (byte offsets, 128-aligned)
 constexpr int sB1 = 0;                          // W1   [64][48]
 constexpr int sB2 = sB1 + kHid * kIn * 2;       // W2   [64][64]
 constexpr int sB3 = sB2 + kHid * kHid * 2;      // W3   [16][64]
-constexpr int sB4 = sB3 + kOutP * kHid * 2;     // W3^T [64][16]
-constexpr int sB5 = sB4 + kHid * kOutP * 2;     // W2^T [64][64]
-constexpr int sA1 = sB5 + kHid * kHid * 2;      // X    [128][48]
+constexpr int sA1 = sB3 + kOutP * kHid * 2;     // X    [128][48]
 constexpr int sA2 = sA1 + kRows * kIn * 2;      // H1   [128][64]
 constexpr int sA3 = sA2 + kRows * kHid * 2;     // H2   [128][64]
-constexpr int sA4 = sA3 + kRows * kHid * 2;     // dOut [128][16]
-constexpr int sA5 = sA4 + kRows * kOutP * 2;    // dZ2  [128][64]
-constexpr int kTileSmem = sA5 + kRows * kHid * 2;
+constexpr int kTileSmem = sA3 + kRows * kHid * 2;
 
 // shared-memory plan of the inference kernel: weights, one input tile, one hidden tile
 // (H1, then H2 over it once the second GEMM has read H1) and the biases in FP32
@@ -59,11 +55,6 @@ __device__ __forceinline__ void put_bf16(unsigned char *base, uint32_t r, uint32
 {
     *reinterpret_cast<__nv_bfloat16 *>(base + tc::kmajor_offset(r, k, K)) = __float2bfloat16_rn(v);
 }
-__device__ __forceinline__ float get_bf16(const unsigned char *base, uint32_t r, uint32_t k, uint32_t K)
-{
-    return __bfloat162float(*reinterpret_cast<const __nv_bfloat16 *>(base + tc::kmajor_offset(r, k, K)));
-}
-
 // 8 consecutive values k0 .. k0+7 (k0 a multiple of 8) of row r: one 16-byte store, since
 // they form one row of a core matrix
 __device__ __forceinline__ void put_bf16x8(unsigned char *base, uint32_t r, uint32_t k0, uint32_t K, const float *v)
@@ -76,6 +67,18 @@ __device__ __forceinline__ void put_bf16x8(unsigned char *base, uint32_t r, uint
         u[i] = *reinterpret_cast<const uint32_t *>(&p);
     }
     *reinterpret_cast<uint4 *>(base + tc::kmajor_offset(r, k0, K)) = w;
+}
+
+__device__ __forceinline__ void get_bf16x8(const unsigned char *base, uint32_t r, uint32_t k0, uint32_t K, float *v)
+{
+    const uint4 w = *reinterpret_cast<const uint4 *>(base + tc::kmajor_offset(r, k0, K));
+    const uint32_t u[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u[i]));
+        v[2 * i] = f.x;
+        v[2 * i + 1] = f.y;
+    }
 }
 
 // weights and biases of the inference kernel
@@ -92,35 +95,24 @@ __device__ __forceinline__ void stage_infer(const float *prm, unsigned char *sm)
     }
 }
 
-// stage the weights (B operands) of the forward pass and, for training, of the backward pass
-__device__ __forceinline__ void stage_weights(const float *prm, unsigned char *sm, bool train)
+// stage the weights (B operands) of the forward kernel
+__device__ __forceinline__ void stage_weights(const float *prm, unsigned char *sm)
 {
     for (int e = threadIdx.x; e < kHid * kIn; e += blockDim.x) put_bf16(sm + sB1, e / kIn, e % kIn, kIn, prm[oW1 + e]);
     for (int e = threadIdx.x; e < kHid * kHid; e += blockDim.x) put_bf16(sm + sB2, e / kHid, e % kHid, kHid, prm[oW2 + e]);
     for (int e = threadIdx.x; e < kOutP * kHid; e += blockDim.x) put_bf16(sm + sB3, e / kHid, e % kHid, kHid, prm[oW3 + e]);
-    if (train) {
-        // W3^T: row i (hidden), column o (output); W2^T: row i (input), column o (output)
-        for (int e = threadIdx.x; e < kOutP * kHid; e += blockDim.x) {
-            const int o = e / kHid, i = e % kHid;
-            put_bf16(sm + sB4, i, o, kOutP, prm[oW3 + e]);
-        }
-        for (int e = threadIdx.x; e < kHid * kHid; e += blockDim.x) {
-            const int o = e / kHid, i = e % kHid;
-            put_bf16(sm + sB5, i, o, kHid, prm[oW2 + e]);
-        }
-    }
 }
 
 // one GEMM on the tensor cores, waited for by every thread; returns false on time-out
 __device__ __forceinline__ bool run_gemm(uint32_t d_tmem, const unsigned char *A, const unsigned char *B, uint32_t K,
-                                         uint32_t N, uint64_t *mbar, uint32_t &phase, bool accumulate = false)
+                                         uint32_t N, uint64_t *mbar, uint32_t &phase)
 {
     tc::fence_smem_to_async();
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     if (threadIdx.x == 0) {
-        tc::gemm_issue(d_tmem, A, B, K, N, accumulate);
+        tc::gemm_issue(d_tmem, A, K, B, K, K, N);
         tc::commit(mbar);
     }
     // block-uniform result: every thread takes the same path afterwards

@@ -34,10 +34,11 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
            (uint64_t((sbo >> 4) & 0x3FFFu) << 32) | (uint64_t(1) << 46);
 }
 
-// instruction descriptor of kind::f16: D FP32, A and B BF16, both K-major, M x N
-__host__ __device__ constexpr uint32_t idesc_bf16(uint32_t M, uint32_t N)
+// instruction descriptor of kind::f16: D FP32, A and B BF16, M x N, both K-major or (mn) both
+// MN-major
+__host__ __device__ constexpr uint32_t idesc_bf16(uint32_t M, uint32_t N, bool mn = false)
 {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((N >> 3) << 17) | ((M >> 4) << 24);
+    return (1u << 4) | (1u << 7) | (1u << 10) | (mn ? 3u << 15 : 0u) | ((N >> 3) << 17) | ((M >> 4) << 24);
 }
 
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate)
@@ -132,16 +133,31 @@ __device__ __forceinline__ void tmem_ld64(uint32_t taddr, float *v)
     for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// D[128 x N] (+)= A[128 x K] B[N x K]^T; issued by one thread; A, B K-major in shared memory
-__device__ __forceinline__ void gemm_issue(uint32_t d_tmem, const void *A, const void *B, uint32_t K, uint32_t N,
-                                           bool accumulate)
+// D[128 x N] = A[128 x K] B[N x K]^T; issued by one thread; A, B K-major in shared memory, stored
+// with Ka and Kb columns
+__device__ __forceinline__ void gemm_issue(uint32_t d_tmem, const void *A, uint32_t Ka, const void *B, uint32_t Kb, uint32_t K,
+                                           uint32_t N)
 {
     const uint32_t id = idesc_bf16(128, N);
-    const uint32_t sbo = (K / 8) * 128u;
     const uint32_t a0 = smem_addr(A), b0 = smem_addr(B);
     for (uint32_t ks = 0; ks < K / 16; ++ks) {
-        const uint64_t ad = smem_desc(a0 + ks * 256u, 128u, sbo);
-        const uint64_t bd = smem_desc(b0 + ks * 256u, 128u, sbo);
+        const uint64_t ad = smem_desc(a0 + ks * 256u, 128u, (Ka / 8) * 128u);
+        const uint64_t bd = smem_desc(b0 + ks * 256u, 128u, (Kb / 8) * 128u);
+        mma_bf16(d_tmem, ad, bd, id, ks > 0 ? 1u : 0u);
+    }
+}
+
+// D[128 x N] (+)= A^T B over K rows of A [K][Ca] and B [K][Cb], stored as for gemm_issue: read
+// MN-major, core matrices are 128 B apart along the units (stride offset) and a row group's
+// (C/8) * 128 B apart along K (leading offset).  Units of A past Ca give rows of D that mean nothing.
+__device__ __forceinline__ void gemm_issue_mn(uint32_t d_tmem, const void *A, uint32_t Ca, const void *B, uint32_t Cb, uint32_t K,
+                                              uint32_t N, bool accumulate)
+{
+    const uint32_t id = idesc_bf16(128, N, true);
+    const uint32_t a0 = smem_addr(A), b0 = smem_addr(B), la = (Ca / 8) * 128u, lb = (Cb / 8) * 128u;
+    for (uint32_t ks = 0; ks < K / 16; ++ks) {
+        const uint64_t ad = smem_desc(a0 + ks * 2u * la, la, 128u);
+        const uint64_t bd = smem_desc(b0 + ks * 2u * lb, lb, 128u);
         mma_bf16(d_tmem, ad, bd, id, (accumulate || ks > 0) ? 1u : 0u);
     }
 }
