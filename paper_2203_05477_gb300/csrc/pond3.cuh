@@ -123,11 +123,6 @@ static __constant__ FacePerm kFacePerm = make_face_perm();
 
 // ------------------------------------------------------------------ parameters
 
-// faces listed in this step, the next one to take, and the tail's CTAs that are through
-struct TailList {
-    unsigned int n, next, ctas, pad;
-};
-
 template <typename R>
 struct Params3 {
     using W = typename FrameWords<R>::word;

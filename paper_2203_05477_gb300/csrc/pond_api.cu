@@ -244,6 +244,7 @@ pond_status setup(pond_state *s)
     const size_t o_xfr2 = take(sizeof(W) * (D + 1) * nxf);
     const size_t o_yfr2 = D == 2 ? take(sizeof(W) * (D + 1) * nyf) : 0;
     const size_t o_clock = take(sizeof(pond::Clock)), o_diag = take(sizeof(pond::Diag));
+    const size_t o_tail = take(sizeof(pond::TailList));
     size_t stage = 4 * size_t(n);
     stage = std::max<size_t>(stage, size_t(NFC + NGC + D + 1) * size_t(n));
     stage = std::max<size_t>(stage, size_t(D + 1) * size_t(nxf + nyf));
@@ -273,6 +274,7 @@ pond_status setup(pond_state *s)
     P.yfr_n = D == 2 ? reinterpret_cast<W *>(s->base + o_yfr2) : nullptr;
     P.clock = reinterpret_cast<pond::Clock *>(s->base + o_clock);
     P.diag = reinterpret_cast<pond::Diag *>(s->base + o_diag);
+    P.tail = reinterpret_cast<pond::TailList *>(s->base + o_tail);
     s->clock = P.clock;
     s->diag = P.diag;
     s->stage = reinterpret_cast<double *>(s->base + o_stage);
@@ -489,6 +491,14 @@ pond_status keep_graph(pond_state *s, cudaGraph_t g, int parity)
     return POND_OK;
 }
 
+// kernels of a step of separate launches: faces (with a tail kernel on FP64 D2Q16 grids without the
+// predictor), cells, the predictor
+template <int D, typename R>
+int step_launches(const pond_state *s)
+{
+    return 2 + (D == 2 && s->learned ? 1 : 0) + (D == 2 && sizeof(R) == 8 && !s->learned && !s->equilibrate ? 1 : 0);
+}
+
 template <int D, typename R>
 pond_status step_impl(pond_state *s, int64_t n_steps)
 {
@@ -505,7 +515,7 @@ pond_status step_impl(pond_state *s, int64_t n_steps)
             CUDA_TRY(cudaStreamEndCapture(s->stream, &g));
             if (pond_status st = keep_graph(s, g, parity)) return st;
         }
-        const int per_step = (s->scheme == POND_SL || fused_step<D, R>(s, false)) ? 1 : 2 + ((D == 2 && s->learned) ? 1 : 0);
+        const int per_step = (s->scheme == POND_SL || fused_step<D, R>(s, false)) ? 1 : step_launches<D, R>(s);
         while (left >= kGraphSteps) {
             CUDA_TRY(cudaGraphLaunch(s->graph_exec[parity], s->stream));
             s->launches += per_step * kGraphSteps;
@@ -515,7 +525,7 @@ pond_status step_impl(pond_state *s, int64_t n_steps)
     for (; left > 0; --left) {
         const int64_t before = s->launches;
         launch_step<D, R>(s);
-        s->launches = before + ((s->scheme == POND_SL || fused_step<D, R>(s, false)) ? 1 : 2 + ((D == 2 && s->learned) ? 1 : 0));
+        s->launches = before + ((s->scheme == POND_SL || fused_step<D, R>(s, false)) ? 1 : step_launches<D, R>(s));
     }
     CUDA_TRY(cudaGetLastError());
     return POND_OK;
@@ -1974,7 +1984,7 @@ pond_status time_grid_variant(pond_state *s, const char *saved, int steps, int w
         pond::launch_cell_any<D, R>(s->cell_v, P, s->stream);
         if (which == 1) CUDA_TRY(cudaEventRecord(ev[2 * k + 1], s->stream));
     }
-    s->launches += int64_t(steps + 1) * (2 + ((D == 2 && s->learned) ? 1 : 0));
+    s->launches += int64_t(steps + 1) * step_launches<D, R>(s);
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaEventSynchronize(ev.back()));
     double sum = 0.0;

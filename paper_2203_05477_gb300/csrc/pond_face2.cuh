@@ -22,12 +22,13 @@
 // few per warp, and would keep whole warps (and, at small sizes, the whole launch) waiting.
 // So a warp goes on pass by pass only while more than coop_faces of its faces need it; the
 // others go to a list that the CTA's warps then work off with 16 lanes per face, one lane per
-// population (coop_tail).
+// population (coop_tail).  In FP64 (without the predictor) the list is the whole grid's and a kernel of its
+// own works it off (lane_tail_kernel).
 //
 // Measured (GB300, us a launch; before: the best of the node-by-node tiles, that is 8 x 8 with
 // shared scratch in FP32 and 8 x 8 in FP64, and the 32 x 4 tile that was the default): FP32 quadrants
 // 1024^2 290 (328, default 446), shocked interface 1001 x 253 with minmod 110 (130, 186); FP64
-// quadrants 256^2 1310 (3208).  FP32 issues 143 M instructions where the node-by-node tile issued 252 M,
+// quadrants 256^2 965 with the tail kernel (3208; 1310 with the CTA's own tail).  FP32 issues 143 M instructions where the node-by-node tile issued 252 M,
 // at 49% of the issue slots with 12 warps per SM: a packed multiply-add with three different
 // register pairs takes four cycles of the register file (two with a repeated operand), the
 // dependent-instruction waits come next (1.6 of 6 cycles), then the loads around the pass.  Four CTAs
@@ -373,12 +374,20 @@ __device__ __forceinline__ void lane_pass(const LaneCell<V> *base, int dir, int 
 // a pass by 16 lanes: R words of a group's part of shared memory (8 moved cells of 16
 // coefficients, padded against bank conflicts, and the 16 moments)
 constexpr int kCoopCell = 17, kCoopWords = 8 * kCoopCell + 16;
+// FP64 without the predictor: the faces that their warps leave go to a list of the whole grid, which
+// lane_tail_kernel works off, instead of to the CTA's own.
+template <typename R, int MODE>
+__host__ __device__ constexpr bool chip_tail() { return sizeof(R) == 8 && MODE == FACE_PLAIN; }
+constexpr int kTailThreads = 128, kTailCtas = 2;
+
 // A warp with at most this many unfinished faces hands them over.  FP32 (64 faces a warp): a pass of
 // the warp costs about as much as one of 12 faces by groups (quadrants 1024^2: 0.302 / 0.290 /
 // 0.289 ms a launch for 6 / 12 / 20; shocked interface 1001 x 253: 0.113 / 0.110 / 0.116).  FP64 (32
-// faces): a pass takes 64 cycles per instruction however few lanes need it, so more go over
-// (quadrants 256^2, 8 x 8 tiles: 1.64 / 1.48 / 1.38 ms for 6 / 12 / 20).
-template <typename R> __host__ __device__ constexpr int coop_faces() { return sizeof(R) == 4 ? 12 : 20; }
+// faces): a pass takes 64 cycles per instruction however few lanes need it, so more go over, and
+// all of them where the whole chip takes them (quadrants 49 x 583 / 64^2 / 256^2, us a launch with
+// the tail: 884 / 495 / 994 for 20, 718 / 375 / 969 for 31; smooth 300^2 2241 and 2266).
+template <typename R, int MODE>
+__host__ __device__ constexpr int coop_faces() { return sizeof(R) == 4 ? 12 : (chip_tail<R, MODE>() ? 31 : 20); }
 // how a face came to the list: to be passed again from its next frame, or after a pass that
 // defined no frame (COOP_BAD), or after a learned prediction that did not hold (COOP_FAIL)
 enum { COOP_BAD = 1, COOP_FAIL = 2, COOP_LEARNED = 4 };
@@ -446,11 +455,61 @@ struct FaceCount {
     unsigned int iters, nonconv, fallbacks, nonphys;
 };
 
+// a warp's or a thread's counts of faces into the diagnostics
+__device__ __forceinline__ void count_faces(Diag *diag, const FaceCount &fc, unsigned int solves)
+{
+    using U = unsigned long long;
+    atomicAdd(&diag->face_iters, U(fc.iters));
+    if (solves) atomicAdd(&diag->face_solves, U(solves));
+    if (fc.nonconv) { atomicAdd(&diag->nonconv, U(fc.nonconv)); atomicOr(&diag->flags, FLAG_NOT_CONVERGED); }
+    if (fc.fallbacks) atomicAdd(&diag->fallbacks, U(fc.fallbacks));
+    if (fc.nonphys) { atomicAdd(&diag->nonphys, U(fc.nonphys)); atomicOr(&diag->flags, FLAG_NONPHYSICAL); }
+}
+
 // plane of coefficient k (hidx order, normal first) of a y-face
 __host__ __device__ constexpr int lane_plane_y(int k)
 {
     const int t[10] = {0, 2, 1, 5, 4, 3, 9, 8, 7, 6};
     return t[k];
+}
+
+// Population (m, n) of the lane reconstructed from the stencil cells in the pass frame (cells), and the
+// 16 moments of the group's populations, one per lane; every lane of the warp calls it
+template <typename R>
+__device__ __forceinline__ R coop_moments(const R *cells, int q, const R *basis, const R *weight, R un, R utn, R h_dn, R h_dt, int limiter)
+{
+    const bool left = un > R(0);
+    auto eval = [&](int s, R &f, R &g) {
+        const R *c = cells + s * kCoopCell;
+        f = c[0];
+        g = c[10];
+#pragma unroll
+        for (int k = 1; k < 10; ++k) f = vfma(c[k], basis[k], f);
+#pragma unroll
+        for (int k = 1; k < 6; ++k) g = vfma(c[10 + k], basis[k], g);
+    };
+    R fu, gu, fl, gl, fh, gh, fm, gm, fp, gp;
+    eval(left ? 1 : 2, fu, gu);
+    eval(left ? 0 : 1, fl, gl);
+    eval(left ? 2 : 3, fh, gh);
+    eval(left ? 4 : 6, fm, gm);
+    eval(left ? 5 : 7, fp, gp);
+    R offn = (left ? R(0.5) : R(-0.5)) - un * h_dn, offt = -utn * h_dt;
+    if (limiter == 1) {
+        fu = vfma(offt, vminmod(fu - fm, fp - fu), vfma(offn, vminmod(fu - fl, fh - fu), fu));
+        gu = vfma(offt, vminmod(gu - gm, gp - gu), vfma(offn, vminmod(gu - gl, gh - gu), gu));
+    } else {
+        offn *= R(2);
+        offt *= R(2);
+        fu = vfma(offt, vanleer_half(fu - fm, fp - fu), vfma(offn, vanleer_half(fu - fl, fh - fu), fu));
+        gu = vfma(offt, vanleer_half(gu - gm, gp - gu), vfma(offn, vanleer_half(gu - gl, gh - gu), gu));
+    }
+    R c[16];
+#pragma unroll
+    for (int k = 0; k < 10; ++k) c[k] = weight[k] * fu;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) c[10 + k] = weight[k] * gu;
+    return reduce16(c, q);
 }
 
 // Works off the CTA's list of unfinished faces, 16 lanes per face.  Lane q of a group moves
@@ -586,39 +645,7 @@ __device__ __forceinline__ void coop_tail(const Params<2, R> &P, const typename 
         }
         __syncwarp();
         const R un = vfma(sqTl, cm, bna + dn), utn = vfma(sqTl, cn, bta + dt);
-        const bool left = un > R(0);
-        auto eval = [&](int s, R &f, R &g) {
-            const R *c = cells + s * kCoopCell;
-            f = c[0];
-            g = c[10];
-#pragma unroll
-            for (int k = 1; k < 10; ++k) f = vfma(c[k], basis[k], f);
-#pragma unroll
-            for (int k = 1; k < 6; ++k) g = vfma(c[10 + k], basis[k], g);
-        };
-        R fu, gu, fl, gl, fh, gh, fm, gm, fp, gp;
-        eval(left ? 1 : 2, fu, gu);
-        eval(left ? 0 : 1, fl, gl);
-        eval(left ? 2 : 3, fh, gh);
-        eval(left ? 4 : 6, fm, gm);
-        eval(left ? 5 : 7, fp, gp);
-        const R h_dn = dir ? KC.h_dy : KC.h_dx, h_dt = dir ? KC.h_dx : KC.h_dy;
-        R offn = (left ? R(0.5) : R(-0.5)) - un * h_dn, offt = -utn * h_dt;
-        if (P.limiter == 1) {
-            fu = vfma(offt, vminmod(fu - fm, fp - fu), vfma(offn, vminmod(fu - fl, fh - fu), fu));
-            gu = vfma(offt, vminmod(gu - gm, gp - gu), vfma(offn, vminmod(gu - gl, gh - gu), gu));
-        } else {
-            offn *= R(2);
-            offt *= R(2);
-            fu = vfma(offt, vanleer_half(fu - fm, fp - fu), vfma(offn, vanleer_half(fu - fl, fh - fu), fu));
-            gu = vfma(offt, vanleer_half(gu - gm, gp - gu), vfma(offn, vanleer_half(gu - gl, gh - gu), gu));
-        }
-        R c[16];
-#pragma unroll
-        for (int k = 0; k < 10; ++k) c[k] = weight[k] * fu;
-#pragma unroll
-        for (int k = 0; k < 6; ++k) c[10 + k] = weight[k] * gu;
-        mom[q] = reduce16(c, q);
+        mom[q] = coop_moments<R>(cells, q, basis, weight, un, utn, dir ? KC.h_dy : KC.h_dx, dir ? KC.h_dx : KC.h_dy, P.limiter);
         __syncwarp();
         R rho = mom[0], du_n, du_t, T1;
         moments_frame<R>(rho, mom[1], mom[2], mom[3], mom[5], mom[10], Tl, sq, Cv, du_n, du_t, T1);
@@ -766,7 +793,7 @@ lane_face_kernel(const Params<2, R> P)
     using V = typename VecOf<R>::type;
     using W = typename FrameWords<R>::word;
     constexpr int L = VecOf<R>::lanes;
-    constexpr bool LEARNED = MODE == FACE_LEARNED;
+    constexpr bool LEARNED = MODE == FACE_LEARNED, CHIP = chip_tail<R, MODE>();
     constexpr int TX = VT::TX, TY = VT::TY, TH = TY / L;   // TH rows of threads; lane l is TH rows up
     constexpr int BX = TX + 3, BH = TH + 3, NT = lane_threads<R, VT>();
     static_assert(TY % L == 0 && (TX * TH) % 32 == 0 && NT <= 256, "whole warps per face direction");
@@ -775,9 +802,10 @@ lane_face_kernel(const Params<2, R> P)
     unsigned char *scratch = lane_smem + sizeof(LaneCell<V>) * BH * BX;
     using Scr = LaneScratch<V, NT>;
     const Scr scr{(unsigned)__cvta_generic_to_shared(scratch) + threadIdx.x * 16u};
-    __shared__ CoopItem items[NT * L];
+    __shared__ CoopItem items[CHIP ? 1 : NT * L];
     __shared__ int n_items, next_item;
     if (threadIdx.x == 0) n_items = next_item = 0;
+    unsigned int n_act = 0;   // faces finished by the warp itself, or listed for the grid's tail
 
     const Clock &K = *P.clock;
     const double step_dt = K.dt;   // 0: t_end reached, the step is a no-op (tested after the staging loads)
@@ -930,7 +958,7 @@ lane_face_kernel(const Params<2, R> P)
         }
         unsigned left_over = __popc(__ballot_sync(0xffffffffu, run[0]));
         if constexpr (L > 1) left_over += __popc(__ballot_sync(0xffffffffu, run[L - 1]));
-        const bool go_on = left_over > coop_faces<R>();
+        const bool go_on = left_over > coop_faces<R, MODE>();
         bool store = go_on;
 #pragma unroll
         for (int l = 0; l < L; ++l) {
@@ -938,7 +966,24 @@ lane_face_kernel(const Params<2, R> P)
             if (flags[l] < 0) continue;
             store = true;
             active[l] = false;   // finished by the tail
-            items[atomicAdd(&n_items, 1)] = {int(threadIdx.x) | (l << 8) | (flags[l] << 16), iters[l]};
+            if constexpr (!CHIP) items[atomicAdd(&n_items, 1)] = {int(threadIdx.x) | (l << 8) | (flags[l] << 16), iters[l]};
+        }
+        if constexpr (CHIP) {
+            // the face's frames go into its own output planes, then it takes a place in the list
+            const unsigned lists = __ballot_sync(0xffffffffu, flags[0] >= 0);
+            if (lists) {
+                unsigned at = 0;
+                if ((threadIdx.x & 31) == 0) at = atomicAdd(&P.tail->n, __popc(lists));
+                at = __shfl_sync(0xffffffffu, at, 0) + __popc(lists & ((1u << (threadIdx.x & 31)) - 1u));
+                if (flags[0] >= 0) {
+                    const long long f = face(0);
+                    R *o = (dir == 0 ? P.xf : P.yf) + f;
+                    o[0] = vget(nn, 0); o[nf] = vget(nt, 0); o[2 * nf] = vget(vn, 0); o[3 * nf] = vget(vt, 0);
+                    o[4 * nf] = vget(nT, 0); o[5 * nf] = vget(vT, 0); o[6 * nf] = R(iters[0]);
+                    P.tail_items()[at] = (unsigned long long)f | (unsigned long long)dir << kTailDirShift | (flags[0] & COOP_BAD ? kTailBad : 0ull);
+                    ++n_act;
+                }
+            }
         }
         if (store) {
             scr.put(S_DL, nn, nt);
@@ -948,7 +993,6 @@ lane_face_kernel(const Params<2, R> P)
         if (!go_on) break;
     }
     FaceCount fc{0, 0, 0, 0};
-    unsigned int n_act = 0;   // faces finished by the warp itself
     bool write = false;
 #pragma unroll
     for (int l = 0; l < L; ++l) {
@@ -983,22 +1027,223 @@ lane_face_kernel(const Params<2, R> P)
             Frm[2 * nf + f] = fr_word(vget(T1, l));
         }
     }
-    __syncthreads();
-    const int count = n_items;
-    if (count > 0) coop_tail<R, MODE, VT>(P, ut, tile, scratch, items, count, &next_item, fc);
+    int count = 0;
+    if constexpr (!CHIP) {
+        __syncthreads();
+        count = n_items;
+        if (count > 0) coop_tail<R, MODE, VT>(P, ut, tile, scratch, items, count, &next_item, fc);
+    }
     fc.iters = warp_sum_count(fc.iters);
     fc.nonconv = warp_sum_count(fc.nonconv);
     fc.fallbacks = warp_sum_count(fc.fallbacks);
     fc.nonphys = warp_sum_count(fc.nonphys);
     if (threadIdx.x == 0) n_act += count;
     n_act = warp_sum_count(n_act);
-    if ((threadIdx.x & 31) == 0 && (n_act || fc.iters)) {
-        using U = unsigned long long;
-        atomicAdd(&P.diag->face_iters, U(fc.iters));
-        atomicAdd(&P.diag->face_solves, U(n_act));
-        if (fc.nonconv) { atomicAdd(&P.diag->nonconv, U(fc.nonconv)); atomicOr(&P.diag->flags, FLAG_NOT_CONVERGED); }
-        if (fc.fallbacks) atomicAdd(&P.diag->fallbacks, U(fc.fallbacks));
-        if (fc.nonphys) { atomicAdd(&P.diag->nonphys, U(fc.nonphys)); atomicOr(&P.diag->flags, FLAG_NONPHYSICAL); }
+    if ((threadIdx.x & 31) == 0 && (n_act || fc.iters)) count_faces(P.diag, fc, n_act);
+}
+
+// Works off the grid's list of unfinished faces (FP64), 16 lanes per face and two faces a warp: the form
+// of coop_tail, with lane q < 8 holding stencil cell q in registers and velocities relative to the face's
+// own predictor frame.  Faces that take many passes lie together (a shock crosses a few tiles), and
+// FP64 needs a warp on every sub-partition: the list spreads them over the chip.  Measured (GB300, us a
+// launch of face and tail; before: each CTA its own list): quadrants 256^2 965 (1310), 64^2 375 (1007),
+// 49 x 583 720 (1117), interface 401 x 201 1066 (1388), smooth 300^2 2260 (2222).  Two CTAs per SM (three:
+// 5% slower).  Two warps a face, f and g apart, halve the chain of a pass but cost twice the issue:
+// 850 at 49 x 583, 1105 at 256^2.
+template <typename R>
+__global__ void __launch_bounds__(kTailThreads)
+lane_tail_kernel(const Params<2, R> P)
+{
+    using W = typename FrameWords<R>::word;
+    using V = typename VecOf<R>::type;
+    static_assert(VecOf<R>::lanes == 1, "FP64");
+    __shared__ R words[kTailThreads / 16][kCoopWords];
+    const unsigned full = 0xffffffffu;
+    const int q = threadIdx.x & 15, lead = threadIdx.x & 16, m = q >> 2, n = q & 3;
+    R *cells = words[threadIdx.x >> 4], *mom = cells + 8 * kCoopCell;
+    const unsigned int count = P.tail->n;
+    const StepC<R> &KC = step_c<R>(*P.clock);
+    const NodeTab<R> &tab = node_tab<R>();
+    const R Cv = P.Cv_r, tol = P.tol_r, cm = tab.c[m], cn = tab.c[n];
+    R basis[10], weight[10];   // as in coop_tail
+#pragma unroll
+    for (int a = 0; a <= 3; ++a)
+#pragma unroll
+        for (int b = 0; a + b <= 3; ++b) {
+            basis[hidx(a, b)] = tab.hen[m][a] * tab.hen[n][b];
+            weight[hidx(a, b)] = tab.whe[m][a] * tab.whe[n][b];
+        }
+    FaceCount fc{0, 0, 0, 0};
+    int dir = 0, iters = 0, fallbacks = 0;
+    long long f = 0, nf = 0;
+    LaneCell<V> cell{};
+    cell.sym[4] = R(1);   // (a group without a face passes over a cell at rest)
+    W ref[2] = {};
+    R una = R(0), uta = R(0), dn = R(0), dt = R(0), Tl = R(1), vn = R(0), vt = R(0), vT = R(1);
+    bool live = false, have = false, done = false, restarted = false, redo = false, bad = false;
+    auto take = [&]() {
+        unsigned int item = 0;
+        if (q == 0) item = atomicAdd(&P.tail->next, 1u);
+        item = __shfl_sync(lead ? 0xffff0000u : 0x0000ffffu, item, lead);
+        live = item < count;
+        if (!live) return;
+        const unsigned long long it = P.tail_items()[item];
+        dir = int(it >> kTailDirShift) & 1;
+        f = (long long)(it & ((1ull << kTailDirShift) - 1));
+        bad = (it & kTailBad) != 0;
+        nf = dir == 0 ? P.nxf() : P.nyf();
+        const long long w = dir == 0 ? P.nx + 1 : P.nx, fj = f / w, fi = f - fj * w;
+        const R *o = (dir == 0 ? P.xf : P.yf) + f;
+        dn = o[0]; dt = o[nf]; vn = o[2 * nf]; vt = o[3 * nf]; Tl = o[4 * nf]; vT = o[5 * nf];
+        iters = int(o[6 * nf]);
+        fallbacks = bad ? 1 : 0;
+        have = !bad || iters > 1;
+        done = restarted = redo = false;
+        const W *Frm = dir == 0 ? P.xfr : P.yfr;
+        ref[0] = Frm[f];
+        ref[1] = Frm[nf + f];
+        una = R(fr_lead(dir ? ref[1] : ref[0]));
+        uta = R(fr_lead(dir ? ref[0] : ref[1]));
+        if (q < 8) {
+            const int on = q < 4 ? q - 2 : (q < 6 ? -1 : 0), ot = q < 4 ? 0 : ((q & 1) ? 1 : -1);
+            stage_any<R, V>(P, fi + (dir ? ot : on), fj + (dir ? on : ot), KC.cp, KC.ce, ref, 0, cell);
+            // in face axes
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                const R x = cell.ax[0][k], y = cell.ax[1][k];
+                cell.ax[0][k] = dir ? y : x;
+                cell.ax[1][k] = dir ? x : y;
+            }
+        }
+    };
+    take();
+    for (;;) {
+        __syncwarp();
+        if (!__any_sync(full, live)) break;
+        // once: the frame of the pooled conserved moments of the eight stencil cells (every lane sums)
+        R r = cell.sym[0], mn = r * cell.ax[0][5], mt = r * cell.ax[1][5];
+        R e = r * (Cv * cell.sym[4] + R(0.5) * (cell.ax[0][5] * cell.ax[0][5] + cell.ax[1][5] * cell.ax[1][5]));
+        if (__any_sync(full, live && bad)) {
+#pragma unroll
+            for (int s = 1; s < 8; s <<= 1) {
+                r += __shfl_xor_sync(full, r, s);
+                mn += __shfl_xor_sync(full, mn, s);
+                mt += __shfl_xor_sync(full, mt, s);
+                e += __shfl_xor_sync(full, e, s);
+            }
+            const int from = lead;   // the sums of lanes 0 .. 7 of the group
+            r = __shfl_sync(full, r, from) * R(0.125);
+            mn = __shfl_sync(full, mn, from) * R(0.125);
+            mt = __shfl_sync(full, mt, from) * R(0.125);
+            e = __shfl_sync(full, e, from) * R(0.125);
+        }
+        if (live && bad) {
+            bad = false;
+            if (!restarted && iters < P.max_iter) {
+                restarted = true;
+                dn = mn / r;
+                dt = mt / r;
+                Tl = (e - R(0.5) * (mn * mn + mt * mt) / r) / (Cv * r);
+            } else {
+                // stopped by a pass without a frame: the last valid one over again, if any
+                redo = true;
+                dn = vn;
+                dt = vt;
+                Tl = vT;
+            }
+        }
+        // ---- the pass
+        const R invTl = vrcp(Tl), rsqTl = vsqrt(invTl), sqTl = Tl * rsqTl, sq = vsqrt(Tl);
+        if (q < 8) {
+            const R *cx = cell.ax[0], *cy = cell.ax[1];
+            const Move2<R> M(cell.sym[4], cx[5], cy[5], Tl, invTl, rsqTl, dn, dt);
+            R F[10], G[6];
+            M.f(cell.sym[0], cx[0], cell.sym[1], cy[0], cx[1], cx[2], cy[2], cy[1], F);
+            M.g(cell.sym[2], cx[3], cy[3], cx[4], cell.sym[3], cy[4], G);
+            R *o = cells + q * kCoopCell;
+#pragma unroll
+            for (int k = 0; k < 10; ++k) o[k] = F[k];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) o[10 + k] = G[k];
+        }
+        __syncwarp();
+        mom[q] = coop_moments<R>(cells, q, basis, weight, vfma(sqTl, cm, una + dn), vfma(sqTl, cn, uta + dt),
+                                 dir ? KC.h_dy : KC.h_dx, dir ? KC.h_dx : KC.h_dy, P.limiter);
+        __syncwarp();
+        R rho = mom[0], du_n, du_t, T1;
+        moments_frame<R>(rho, mom[1], mom[2], mom[3], mom[5], mom[10], Tl, sq, Cv, du_n, du_t, T1);
+        if (!live) continue;
+        bool finished = redo;
+        if (!redo) {
+            ++iters;
+            const bool ok = T1 > R(0) && isfinite(T1) && isfinite(rho) && isfinite(du_n) && isfinite(du_t);
+            if (ok) {
+                have = true;
+                vn = dn;
+                vt = dt;
+                vT = Tl;
+                if (P.fixed_iters > 0) done = iters >= P.fixed_iters;
+                else done = fabs(T1 - Tl) <= tol * Tl && fabs(du_n) <= tol * sq && fabs(du_t) <= tol * sq;
+                finished = done || iters >= P.max_iter;
+                if (!finished) {
+                    dn += du_n;
+                    dt += du_t;
+                    Tl = T1;
+                }
+            } else {
+                ++fallbacks;
+                if (!have && (restarted || iters >= P.max_iter)) finished = true;
+                else bad = true;
+            }
+        }
+        if (!finished) continue;
+        // ---- the face's result
+        R *Fout = dir == 0 ? P.xf : P.yf, *Gout = dir == 0 ? P.xg : P.yg;
+        W *Frm = dir == 0 ? P.xfr : P.yfr;
+        const unsigned half = lead ? 0xffff0000u : 0x0000ffffu;
+        R v = R(__longlong_as_double(0x7ff8000000000000ll));
+        if (have) {
+            R Phi[10], Psi[6], Fo[10], Go[6];
+#pragma unroll
+            for (int k = 0; k < 10; ++k) Phi[k] = mom[k];
+#pragma unroll
+            for (int k = 0; k < 6; ++k) Psi[k] = mom[10 + k];
+            face_populations<R>(Phi, Psi, Tl, rho, du_n, du_t, T1, KC.wb, KC.we, P.Cvh_r, Fo, Go);
+            __syncwarp(half);
+            if (q == 0) {
+#pragma unroll
+                for (int k = 0; k < 10; ++k) mom[k] = Fo[k];
+#pragma unroll
+                for (int k = 0; k < 6; ++k) mom[10 + k] = Go[k];
+                const R fn = dn + du_n, ft = dt + du_t;
+                Frm[f] = fr_add(ref[0], dir ? ft : fn);
+                Frm[nf + f] = fr_add(ref[1], dir ? fn : ft);
+                Frm[2 * nf + f] = fr_word(T1);
+            }
+            __syncwarp(half);
+            v = mom[q];
+        } else if (q == 0) {
+            fr_store(Frm[2 * nf + f], double(v));
+        }
+        const int k = q < 10 ? q : q - 10;
+        int pl = k;
+        if (dir) pl = k == 0 || k == 4 ? k : (k < 3 ? 3 - k : (k < 6 ? 8 - k : 15 - k));   // axes exchanged
+        (q < 10 ? Fout : Gout)[pl * nf + f] = v;
+        if (q == 0) {
+            fc.iters += iters;
+            fc.fallbacks += fallbacks;
+            fc.nonconv += done ? 0 : 1;
+            fc.nonphys += have ? 0 : 1;
+        }
+        take();
+    }
+    if (q == 0 && fc.iters) count_faces(P.diag, fc, 0);
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(&P.tail->ctas, 1u) == gridDim.x - 1) {
+        // every CTA has taken its last ticket: empty the list
+        P.tail->n = 0u;
+        P.tail->next = 0u;
+        P.tail->ctas = 0u;
     }
 }
 

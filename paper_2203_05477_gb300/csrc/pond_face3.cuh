@@ -453,17 +453,6 @@ __device__ __forceinline__ void pass3(const R *base, const FaceAxes3<R> &ax, con
     }
 }
 
-// a warp's or a thread's counts of faces into the diagnostics
-__device__ __forceinline__ void count_faces(Diag *diag, const FaceCount &fc, unsigned int solves)
-{
-    using U = unsigned long long;
-    atomicAdd(&diag->face_iters, U(fc.iters));
-    if (solves) atomicAdd(&diag->face_solves, U(solves));
-    if (fc.nonconv) { atomicAdd(&diag->nonconv, U(fc.nonconv)); atomicOr(&diag->flags, FLAG_NOT_CONVERGED); }
-    if (fc.fallbacks) atomicAdd(&diag->fallbacks, U(fc.fallbacks));
-    if (fc.nonphys) { atomicAdd(&diag->nonphys, U(fc.nonphys)); atomicOr(&diag->flags, FLAG_NONPHYSICAL); }
-}
-
 // the frame of a pass's moments relative to the pass frame
 template <typename R>
 __device__ __forceinline__ bool moments_frame3(const R *p, const R *g, R Tl, R sq, R Cv, R &rho, R *du, R &T1)
@@ -530,10 +519,8 @@ inline int tail3_faces(long long faces, int sms, int fixed_iters)
 // R words of a warp in the tail kernel: the 12 stencil cells as staged, the same in the pass frame, and
 // 32 moments
 constexpr int kTailCell3 = 31, kTailWords3 = 12 * kCell3 + 12 * kTailCell3 + 32, kTailThreads3 = 128;
-// a listed face: its index, with the axis and whether its last pass defined no frame above; the
-// passes so far, its next frame and its last valid one wait in its own output planes
-constexpr unsigned long long kTailBad = 1ull << 62;
-constexpr int kTailDirShift = 60;
+// (of a listed face the passes so far, its next frame and its last valid one wait in its own output
+// planes)
 
 // the sum over the warp of each of c[0..31]; lane q returns that of c[q]
 template <typename R>

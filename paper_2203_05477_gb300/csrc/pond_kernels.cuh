@@ -176,6 +176,15 @@ struct StageMaps {
     const void *key;
 };
 
+// The list of the faces that a face kernel leaves to its tail kernel: faces listed in this step, the
+// next one to take, and the tail's CTAs that are through
+struct TailList {
+    unsigned int n, next, ctas, pad;
+};
+// a listed face: its index, with the axis and whether its last pass defined no frame above
+constexpr unsigned long long kTailBad = 1ull << 62;
+constexpr int kTailDirShift = 60;
+
 template <int D, typename R>
 struct Params {
     static constexpr int NFC = NCoef<D, 3>::value;   // f coefficients per face
@@ -223,9 +232,14 @@ struct Params {
                                       // previous frame; larger moves may reach another fixed point)
     unsigned int *mlp_err;
     int sms;                          // SMs of the device (grid sizes of the grid-stride kernels)
+    TailList *tail;                   // D2Q16 in FP64: the faces left to the tail kernel (items: tail_items())
     // host memory: tensor maps of the two state buffers for the TMA-staged face variant (null
     // where the grid does not allow them); read by the launcher, never by a kernel
     const StageMaps *stage_maps;
+    // the list's items, one for each face at most, lie in the planes of the learned predictions, which
+    // the steps without the predictor leave alone: 24 (nx + 1) ny bytes or more in FP64, and the
+    // faces number (nx + 1) ny + nx (ny + 1) <= 3 (nx + 1) ny
+    __device__ unsigned long long *tail_items() const { return reinterpret_cast<unsigned long long *>(xlr); }
     __host__ __device__ long long ncell() const { return nx * ny; }
     __host__ __device__ long long nxf() const { return (nx + 1) * ny; }
     __host__ __device__ long long nyf() const { return nx * (ny + 1); }

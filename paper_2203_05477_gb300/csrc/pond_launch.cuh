@@ -26,7 +26,7 @@ struct VList {
 // D2Q16: the lane kernel (pond_face2.cuh) in tiles that keep whole warps on one direction; us a
 // launch on the 1024^2 quadrants in FP32: 16 x 8 / 3 CTAs per SM 290, 32 x 4 / 3 302, 16 x 8 / 2 318 (the
 // 1001 x 253 interface: 110, 107, 117), against 328-380 for the node-by-node tiles kept below for
-// comparison; FP64 256^2: 8 x 4 / 4 1314, 8 x 8 / 2 1362, 16 x 4 / 2 1401.
+// comparison; FP64 256^2 with the tail kernel: 8 x 4 / 4 961, 8 x 8 / 2 950, 16 x 4 / 2 1330.
 template <int D, typename R>
 struct FaceList;
 template <>
