@@ -1212,6 +1212,7 @@ pond_status pond_init(const pond_grid *grid, pond_velset velset, double gamma, d
     if (st == POND_OK) st = reset_clock(s);
     if (st != POND_OK) { pond_destroy(s); return st; }
     if (D == 1 && s->scheme == POND_FV) s->tube_v = 1 + pond::chunk_default(s->grid.nx, s->sms);
+    if (D == 2 && s->prec == POND_FP32) s->face_v = pond::face2_default(s->grid.nx, s->grid.ny, s->sms);
     s->learned = D == 2 && opts->learned != 0;
     if (s->learned) {
         if (s->prec == POND_FP32) params_of<2, float>(s).use_learned = 1;
@@ -1907,6 +1908,16 @@ std::string tune_key(const pond_state *s)
         std::snprintf(buf, sizeof(buf), "%s|sm%d|D%d|%s|%lldx%lld|learned%d", prop.name, prop.multiProcessorCount, s->D,
                       s->prec == POND_FP32 ? "fp32" : "fp64", (long long)s->grid.nx, (long long)s->grid.ny,
                       s->learned ? 1 : 0);
+    // a choice is an index into the variants' list: the key holds a hash (FNV-1a) of their names, so an
+    // entry made with another list does not match
+    unsigned long long h = 0xcbf29ce484222325ull;
+    for (int i = 0; i < pond_variant_count(s); ++i)
+        for (const char *c = pond_variant_name(s, i); ; ++c) {
+            h = (h ^ (unsigned char)*c) * 0x100000001b3ull;
+            if (!*c) break;
+        }
+    const size_t end = std::strlen(buf);
+    std::snprintf(buf + end, sizeof(buf) - end, "|%016llx", h);
     for (char *c = buf; *c; ++c)
         if (*c == '\t' || *c == '\n') *c = ' ';
     return buf;

@@ -38,6 +38,12 @@ template <>
 struct FaceList<2, double> {
     using type = VList<LaneVariant<8, 4, 4>, LaneVariant<8, 8, 2>, LaneVariant<16, 4, 2>>;
 };
+// The face variant of a D2Q16 FP32 grid before tuning: where every 16 x 8 tile has half an SM to itself, the
+// kernel without the 168-register cap (its tail's passes are the longest chain of a small grid); us a
+// launch capped / uncapped: quadrants 49 x 583 86 / 78, 64^2 94 / 82, 128^2 92 / 79, interface 80 x 229
+// 47 / 44; above the line 300^2 smooth 46 / 48, quadrants 700^2 160 / 169.
+inline int face2_default(long long nx, long long ny, int sms) { return ((nx + 16) / 16) * ((ny + 8) / 8) <= 2ll * sms ? 2 : 0; }
+
 template <typename R>
 struct FaceList<1, R> {
     using type = VList<FaceVariant<1, 128, 1, 1>, FaceVariant<1, 64, 1, 2>, FaceVariant<1, 256, 1, 1>,
