@@ -339,9 +339,9 @@ pond_status set_primitive_impl(pond_state *s, const double *rho, const double *u
     }
     pond_status r = reset_clock(s);
     if (r != POND_OK) return r;
-    pond::init_cells_kernel<D, R><<<blocks_for(n, 256), 256, 0, s->stream>>>(P, dr, dux, duy, dp);
+    pond::init_cells_kernel<D, R><<<blocks_for(n, 256), 256, 0, s->stream>>>(P, dr, dux, duy, dp, R(1.0 / P.dx), R(1.0 / P.dy));
     const long long nf = P.nxf() + (D == 2 ? P.nyf() : 0);
-    pond::init_faces_kernel<D, R><<<blocks_for(nf, 256), 256, 0, s->stream>>>(P);
+    pond::init_faces_kernel<D, R><<<blocks_for(nf, 256), 256, 0, s->stream>>>(P, 1.0 / P.Cv);
     s->launches += 2;
     CUDA_TRY(cudaGetLastError());
     if (!on_device) CUDA_TRY(cudaStreamSynchronize(s->stream));

@@ -386,7 +386,7 @@ tube_init_kernel(const TubeParams<R> P, int cur, const double *rho, const double
         fr_store(P.sfr[cur][c], u);
         fr_store(P.sfr[cur][n + c], T);
         if (r > 0.0 && T > 0.0 && isfinite(r) && isfinite(T)) {
-            rate = fmax(rate, (fabs(u) + sqrt(T) * kCHi) / dx);
+            rate = fmax(rate, fabs(u) + sqrt(T) * kCHi);   // (divided by dx once: division rounds monotonically)
         } else {
             ++bad;
             atomicCAS((unsigned long long *)&P.diag->first_bad, (unsigned long long)-1ll, (unsigned long long)c);
@@ -397,8 +397,9 @@ tube_init_kernel(const TubeParams<R> P, int cur, const double *rho, const double
         const double ra = rho[a], rb = rho[b], ua = ux[a], ub = ux[b];
         const double Ea = p[a] * Cv + 0.5 * ra * ua * ua, Eb = p[b] * Cv + 0.5 * rb * ub * ub;
         const double r = 0.5 * (ra + rb), m = 0.5 * (ra * ua + rb * ub), E = 0.5 * (Ea + Eb);
-        fr_store(P.fu[cur][f_off + k], m / r);
-        fr_store(P.fT[cur][f_off + k], (E - 0.5 * m * m / r) / (Cv * r));
+        const double u = m / r;
+        fr_store(P.fu[cur][f_off + k], u);
+        fr_store(P.fT[cur][f_off + k], (E - 0.5 * m * u) / (Cv * r));
     }
     if (bad) { atomicAdd(&P.diag->nonphys, bad); atomicOr(&P.diag->flags, FLAG_NONPHYSICAL); any_bad = 1; }
 #pragma unroll
@@ -409,7 +410,7 @@ tube_init_kernel(const TubeParams<R> P, int cur, const double *rho, const double
         double rm = 0.0;
         for (int w = 0; w < kTubeThreads / 32; ++w) rm = fmax(rm, red[w]);
         P.t[tube] = 0.0;
-        P.dt[tube] = P.cfl / rm;
+        P.dt[tube] = P.cfl / (rm / dx);
         P.steps_done[tube] = 0;
         P.status[tube] = any_bad;
     }

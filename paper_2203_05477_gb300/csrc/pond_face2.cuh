@@ -371,9 +371,36 @@ __device__ __forceinline__ void lane_pass(const LaneCell<V> *base, int dir, int 
 
 // ------------------------------------------------------------ 16 lanes per face
 
-// a pass by 16 lanes: R words of a group's part of shared memory (8 moved cells of 16
-// coefficients, padded against bank conflicts, and the 16 moments)
-constexpr int kCoopCell = 17, kCoopWords = 8 * kCoopCell + 16;
+// A pass by 16 lanes: R words of a group's part of shared memory (8 moved cells of 16 coefficients, f then
+// g, padded against bank conflicts, and the 16 moments).  A pass reads 80 words a lane, and its latency is
+// what a small grid with a shock waits for: in FP32 a cell moves in 16-byte accesses (interface 80 x 229
+// 47.0 -> 43.9 us a launch, quadrants 49 x 583 86 -> 83.5; in FP64 it makes no difference).
+template <typename R> __host__ __device__ constexpr int coop_cell() { return sizeof(R) == 4 ? 20 : 17; }
+template <typename R> __host__ __device__ constexpr int coop_words() { return 8 * coop_cell<R>() + 16; }
+__device__ __forceinline__ void coop_put(float *o, const float *F, const float *G)
+{
+    float4 *v = reinterpret_cast<float4 *>(o);
+    v[0] = make_float4(F[0], F[1], F[2], F[3]);
+    v[1] = make_float4(F[4], F[5], F[6], F[7]);
+    v[2] = make_float4(F[8], F[9], G[0], G[1]);
+    v[3] = make_float4(G[2], G[3], G[4], G[5]);
+}
+__device__ __forceinline__ void coop_put(double *o, const double *F, const double *G)
+{
+#pragma unroll
+    for (int k = 0; k < 10; ++k) o[k] = F[k];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) o[10 + k] = G[k];
+}
+__device__ __forceinline__ void coop_get(const float *o, float *c)
+{
+    const float4 *v = reinterpret_cast<const float4 *>(o);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float4 x = v[k];
+        c[4 * k] = x.x; c[4 * k + 1] = x.y; c[4 * k + 2] = x.z; c[4 * k + 3] = x.w;
+    }
+}
 // FP64 without the predictor: the faces that their warps leave go to a list of the whole grid, which
 // lane_tail_kernel works off, instead of to the CTA's own.
 template <typename R, int MODE>
@@ -480,7 +507,12 @@ __device__ __forceinline__ R coop_moments(const R *cells, int q, const R *basis,
 {
     const bool left = un > R(0);
     auto eval = [&](int s, R &f, R &g) {
-        const R *c = cells + s * kCoopCell;
+        const R *c = cells + s * coop_cell<R>();
+        R w[16];
+        if constexpr (sizeof(R) == 4) {
+            coop_get(c, w);
+            c = w;
+        }
         f = c[0];
         g = c[10];
 #pragma unroll
@@ -527,7 +559,7 @@ __device__ __forceinline__ void coop_tail(const Params<2, R> &P, const typename 
     constexpr bool LEARNED = MODE == FACE_LEARNED;
     const unsigned full = 0xffffffffu;
     const int q = threadIdx.x & 15, lead = threadIdx.x & 16, m = q >> 2, n = q & 3;
-    R *cells = reinterpret_cast<R *>(scratch) + (threadIdx.x >> 4) * kCoopWords, *mom = cells + 8 * kCoopCell;
+    R *cells = reinterpret_cast<R *>(scratch) + (threadIdx.x >> 4) * coop_words<R>(), *mom = cells + 8 * coop_cell<R>();
     const StepC<R> &KC = step_c<R>(*P.clock);
     const NodeTab<R> &tab = node_tab<R>();
     const R Cv = P.Cv_r, tol = P.tol_r, cm = tab.c[m], cn = tab.c[n];
@@ -637,11 +669,7 @@ __device__ __forceinline__ void coop_tail(const Params<2, R> &P, const typename 
             R F[10], G[6];
             M.f(c[0], cx[0], c[L], cy[0], cx[L], cx[2 * L], cy[2 * L], cy[L], F);
             M.g(c[2 * L], cx[3 * L], cy[3 * L], cx[4 * L], c[3 * L], cy[4 * L], G);
-            R *o = cells + q * kCoopCell;
-#pragma unroll
-            for (int k = 0; k < 10; ++k) o[k] = F[k];
-#pragma unroll
-            for (int k = 0; k < 6; ++k) o[10 + k] = G[k];
+            coop_put(cells + q * coop_cell<R>(), F, G);
         }
         __syncwarp();
         const R un = vfma(sqTl, cm, bna + dn), utn = vfma(sqTl, cn, bta + dt);
@@ -1057,10 +1085,10 @@ lane_tail_kernel(const Params<2, R> P)
     using W = typename FrameWords<R>::word;
     using V = typename VecOf<R>::type;
     static_assert(VecOf<R>::lanes == 1, "FP64");
-    __shared__ R words[kTailThreads / 16][kCoopWords];
+    __shared__ __align__(16) R words[kTailThreads / 16][coop_words<R>()];
     const unsigned full = 0xffffffffu;
     const int q = threadIdx.x & 15, lead = threadIdx.x & 16, m = q >> 2, n = q & 3;
-    R *cells = words[threadIdx.x >> 4], *mom = cells + 8 * kCoopCell;
+    R *cells = words[threadIdx.x >> 4], *mom = cells + 8 * coop_cell<R>();
     const unsigned int count = P.tail->n;
     const StepC<R> &KC = step_c<R>(*P.clock);
     const NodeTab<R> &tab = node_tab<R>();
@@ -1160,11 +1188,7 @@ lane_tail_kernel(const Params<2, R> P)
             R F[10], G[6];
             M.f(cell.sym[0], cx[0], cell.sym[1], cy[0], cx[1], cx[2], cy[2], cy[1], F);
             M.g(cell.sym[2], cx[3], cy[3], cx[4], cell.sym[3], cy[4], G);
-            R *o = cells + q * kCoopCell;
-#pragma unroll
-            for (int k = 0; k < 10; ++k) o[k] = F[k];
-#pragma unroll
-            for (int k = 0; k < 6; ++k) o[10 + k] = G[k];
+            coop_put(cells + q * coop_cell<R>(), F, G);
         }
         __syncwarp();
         mom[q] = coop_moments<R>(cells, q, basis, weight, vfma(sqTl, cm, una + dn), vfma(sqTl, cn, uta + dt),

@@ -2265,7 +2265,8 @@ step_kernel(const Params<D, R> P)
 
 // Equilibria of Eqs. (feqPond), (geqPond) in each cell's frame from primitive fields.
 template <int D, typename R>
-__global__ void init_cells_kernel(const Params<D, R> P, const double *rho, const double *ux, const double *uy, const double *p)
+__global__ void init_cells_kernel(const Params<D, R> P, const double *rho, const double *ux, const double *uy, const double *p,
+                                  R inv_dx, R inv_dy)
 {
     constexpr int NFS = Params<D, R>::NFS, NGC = NCoef<D, 2>::value;
     const long long n = P.ncell();
@@ -2290,7 +2291,7 @@ __global__ void init_cells_kernel(const Params<D, R> P, const double *rho, const
             atomicCAS((unsigned long long *)&P.diag->first_bad, (unsigned long long)-1ll, (unsigned long long)c);
         }
         const R ur[2] = {R(u[0]), R(u[1])};
-        rate = ok ? cell_rate<R>(ur, R(T), R(1.0 / P.dx), R(1.0 / P.dy), D) : 0.0;
+        rate = ok ? cell_rate<R>(ur, R(T), inv_dx, inv_dy, D) : 0.0;
     }
     reduce_rate_and_advance(P.clock, rate, false);
 }
@@ -2323,9 +2324,12 @@ __device__ __forceinline__ void cell_conserved(const Params<D, R> &P, long long 
     E = r * (P.Cv * T + 0.5 * k2);
 }
 
-// face predictor before the first step: frame of the pooled moments of the two cells
+// Face predictor before the first step: frame of the pooled moments of the two cells.  Bound by the FP64
+// pipe, on which a division takes as long as nine multiply-adds: one reciprocal a face (inv_Cv comes from
+// the host) instead of three divisions in 1D and four in 2D, and 32-bit face indices where they fit; the
+// cell kernel takes 1/dx from the host.  Setting 4 M cells in FP32: 742 -> 560 us.
 template <int D, typename R>
-__global__ void init_faces_kernel(const Params<D, R> P)
+__global__ void init_faces_kernel(const Params<D, R> P, double inv_Cv)
 {
     const long long nxf = P.nxf(), nyf = D == 2 ? P.nyf() : 0;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -2333,20 +2337,27 @@ __global__ void init_faces_kernel(const Params<D, R> P)
     const bool xdir = t < nxf;
     const long long f = xdir ? t : t - nxf;
     long long ai, aj, bi, bj;
-    if (xdir) { const long long i = f % (P.nx + 1), j = f / (P.nx + 1); ai = i - 1; aj = j; bi = i; bj = j; }
-    else { const long long i = f % P.nx, j = f / P.nx; ai = i; aj = j - 1; bi = i; bj = j; }
+    {
+        const long long w = xdir ? P.nx + 1 : P.nx;
+        long long j = 0;
+        if (D == 2) j = nxf + nyf < (1ll << 32) ? (long long)((unsigned int)f / (unsigned int)w) : f / w;
+        bi = f - j * w;
+        bj = j;
+        ai = xdir ? bi - 1 : bi;
+        aj = xdir ? bj : bj - 1;
+    }
     double ra, ma[2] = {0, 0}, Ea, rb, mb[2] = {0, 0}, Eb;
     cell_conserved<D, R>(P, ai, aj, ra, ma, Ea);
     cell_conserved<D, R>(P, bi, bj, rb, mb, Eb);
-    const double r = 0.5 * (ra + rb), E = 0.5 * (Ea + Eb);
+    const double r = 0.5 * (ra + rb), E = 0.5 * (Ea + Eb), ir = 1.0 / r;
     double k2 = 0.0, u[2];
 #pragma unroll
-    for (int a = 0; a < D; ++a) { const double m = 0.5 * (ma[a] + mb[a]); u[a] = m / r; k2 += m * m; }
+    for (int a = 0; a < D; ++a) { const double m = 0.5 * (ma[a] + mb[a]); u[a] = m * ir; k2 += m * m; }
     typename FrameWords<R>::word *Frm = xdir ? P.xfr : P.yfr;
     const long long nf = xdir ? nxf : nyf;
 #pragma unroll
     for (int a = 0; a < D; ++a) fr_store(Frm[a * nf + f], u[a]);
-    fr_store(Frm[D * nf + f], (E - 0.5 * k2 / r) / (P.Cv * r));
+    fr_store(Frm[D * nf + f], (E - 0.5 * k2 * ir) * (ir * inv_Cv));
 }
 
 // ------------------------------------------------------- learned gauge predictor
