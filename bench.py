@@ -36,6 +36,7 @@ N_SMS, FP32_LANES = 152, 128
 # ncu dram read + write of one face-kernel launch at 1024^2, for the tile variants measured
 # on the current kernel (profiles/face_kernel_quadrants1024_fp32.md); other variants: null
 FACE_KERNEL_DRAM_BYTES = {
+    "face 16x8 cells, 128 threads, 3 CTA/SM, by upwind side, two faces a thread": 135.430e6 + 133.981e6,
     "face 8x8 cells, 128 threads, 4 CTA/SM, centre cells in shared scratch": 134.708e6 + 136.232e6,
     "face 8x8 cells, 128 threads, 4 CTA/SM, centre cells and moment sums in shared scratch": 134.678e6 + 136.447e6,
     "face 8x8 cells, 128 threads, 4 CTA/SM, centre cells in shared scratch, TMA staging": 134.782e6 + 136.415e6,
@@ -43,11 +44,11 @@ FACE_KERNEL_DRAM_BYTES = {
         134.643e6 + 133.277e6,
 }
 # FP32 operations of one corrector pass at one D2Q16 face (per-face overhead included),
-# counted by ncu on one launch of the headline face variant at 1024^2 (level-2 scratch, TMA
-# staging): FFMA x 2 + FFMA2 x 4 + FMUL + FMUL2 x 2 + FADD + FADD2 x 2 = 8.417 GFLOP over
-# 2,099,200 faces x 1.028 passes (profiles/face_kernel_quadrants1024_fp32.md); used for the
-# ALU roofline.  (The scalar kernel of earlier builds executed 4550 per pass.)
-FLOPS_PER_FACE_PASS = 3900.0
+# counted by ncu on four launches of the face kernel by upwind side at 1024^2: FFMA x 2 + FFMA2 x 4 +
+# FMUL + FMUL2 x 2 + FADD + FADD2 x 2 = 5.601 GFLOP over 2,146,150 face-passes
+# (profiles/face_kernel_quadrants1024_fp32.md); used for the ALU roofline.  (The node-by-node kernel
+# executed 3900 per pass.)
+FLOPS_PER_FACE_PASS = 2610.0
 # algorithmic bytes per cell-update of the FP32 D2Q16 layout: the face kernel reads the
 # cell state (8 + 6 FP32 coefficients + 3 float-float frame words = 80 B) and two face predictors
 # (2 x 24 B) and writes two faces (2 x (16 x 4 + 24) B)
@@ -388,8 +389,8 @@ def bench_tubes(args, n_tubes=4096, seed=0, rank=0):
 
 # executed FP32 FLOP per node-pass of the semi-Lagrangian kernels (FFMA x 2 + FADD + FMUL, packed
 # forms x 2), counted by ncu on the sl_vs_fv workloads: sl_kernel<float> (D1Q4) 4.124 GFLOP per
-# launch over 4.19 M node-passes, sl2_kernel<float> (D2Q16) 41.17 GFLOP over 2.10 M
-SL_FLOPS_PER_NODE_PASS = {1: 983.0, 2: 19.6e3}
+# launch over 4.19 M node-passes, sl2_kernel<float> (D2Q16) 15.31 GFLOP over 2.10 M
+SL_FLOPS_PER_NODE_PASS = {1: 983.0, 2: 7.30e3}
 
 
 def time_schemes(pb, cfl, steps):
@@ -436,9 +437,9 @@ def bench_sl_vs_fv(args, seed=0, rank=0):
 # writes the state.
 D3_FACE_BYTES_PER_CELL = 140 + 3 * 32 + 456
 D3_CELL_BYTES_PER_CELL = 140 + 456 + 140
-# executed FP32 FLOP per face-pass of face3_kernel<float> (FFMA x 2 + FADD + FMUL), counted by
-# ncu on the 64^3 spherical explosion (profiles/face3_kernel_blast64_fp32.md)
-D3_FLOPS_PER_FACE_PASS = 33.6e3
+# executed FP32 FLOP per face-pass of face3_kernel<float> and its tail (FFMA x 2 + FADD + FMUL, packed
+# forms x 2), counted by ncu on the 64^3 spherical explosion (profiles/face3_kernel_blast64_fp32.md)
+D3_FLOPS_PER_FACE_PASS = 17.4e3
 
 
 def bench_d3q64(args, n=128, steps=20, fp64_steps=3, rank=0):
@@ -890,7 +891,7 @@ def main():
         "passes_per_face": face_passes / max(faces, 1),
         "roofline": {"bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
                      "frac": achieved / fp32_peak, "traffic": FACE_KERNEL_DRAM_BYTES.get(variant_names[fv]),
-                     "kernel": ("face_kernel<2,float> (%s)" % variant_names[fv]) if sv == 0 else
+                     "kernel": ("D2Q16 FP32 face kernel (%s)" % variant_names[fv]) if sv == 0 else
                                ("step_kernel<2,float> (%s; faces and cell update)" % [nm for nm in variant_names if nm.startswith("step")][sv]),
                      "peak_source": "152 SMs x 128 FP32 lanes x 2 x %.0f MHz" % sm_mhz,
                      "face_ms": face_ms_avg, "cell_ms": ms_cell / args.steps,

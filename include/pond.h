@@ -271,7 +271,9 @@ pond_status pond_gauge_get_params(pond_state *s, float *params);
  * stream) and waited for: forward pass of n rows x[n][ldx] (first 48 columns) into
  * out[n][16]; and the gradient of the mean squared error against the targets held in
  * columns 48..50 of y[n][ldy] into grad[POND_MLP_PARAMS] and the loss into *loss (device
- * floats).  pond_mlp_gradient allocates its activation scratch with cudaMalloc. */
+ * floats).  pond_mlp_gradient keeps its partial gradients in one of two fixed device arrays
+ * (10 MB each, held by every GPU that loads the library) for the length of the call, and allocates
+ * them with cudaMalloc only while other threads hold both. */
 pond_status pond_mlp_forward(const float *params, const float *x, int ldx, int64_t n, float *out, void *stream);
 pond_status pond_mlp_gradient(const float *params, const float *x, int ldx, const float *y, int ldy, int64_t n,
                               float *grad, float *loss, void *stream);
@@ -319,8 +321,8 @@ pond_status pond_wait_timeout_check(int64_t polls, void *stream);
    The state is copied aside first (one extra device allocation of the state's size, freed
    before returning) and restored afterwards, so tuning leaves the solution unchanged.
    cache_path (may be NULL) names a text file of "key<TAB>face cell tube" lines; a line
-   whose key (device name and SM count, problem kind, precision, size, learned flag)
-   matches this state is used without timing, and a new choice is appended.  File errors
+   whose key (device name and SM count, problem kind, precision, size, learned flag, a hash of
+   the variants' names) matches this state is used without timing, and a new choice is appended.  File errors
    only disable the cache.  Call it outside stream capture.  Errors: INVALID_ARG
    (steps < 1), OOM, CUDA. */
 #define POND_TUNE_MAX 32
@@ -334,8 +336,8 @@ pond_status pond_autotune(pond_state *s, int steps, const char *cache_path, pond
 
 /* Number of variants of this state and the name of variant i: for a 1D or 2D grid, the
    face variants first, then the cell variants, then the whole-step choices (the separate
-   face and cell kernels, then each tile variant of the fused step kernel, which solves a
-   tile's faces and updates its cells in one kernel); for a D3Q64 grid, the face tile
+   face and cell kernels, then each variant of the fused step kernel, which solves a
+   tile's or chunk's faces and updates its cells in one kernel; a 1D grid starts on one of these); for a D3Q64 grid, the face tile
    variants, then the cell block variants; for a batch, the tube variants.  The name
    points to a thread-local buffer ("" when i is out of range). */
 int pond_variant_count(const pond_state *s);
