@@ -491,12 +491,14 @@ pond_status keep_graph(pond_state *s, cudaGraph_t g, int parity)
     return POND_OK;
 }
 
-// kernels of a step of separate launches: faces (with a tail kernel on FP64 D2Q16 grids without the
+// kernels of a step of separate launches: faces (with a tail kernel on D2Q16 grids without the
 // predictor), cells, the predictor
 template <int D, typename R>
 int step_launches(const pond_state *s)
 {
-    return 2 + (D == 2 && s->learned ? 1 : 0) + (D == 2 && sizeof(R) == 8 && !s->learned && !s->equilibrate ? 1 : 0);
+    if (D == 1) return 2;
+    if (s->learned) return 3;
+    return !s->equilibrate && pond::LaneAt<typename pond::FaceList<2, R>::type>::at(s->face_v) ? 3 : 2;
 }
 
 template <int D, typename R>

@@ -21,14 +21,13 @@
 // Nearly every face converges in its first pass, but the faces at shocks take up to max_iter, a
 // few per warp, and would keep whole warps (and, at small sizes, the whole launch) waiting.
 // So a warp goes on pass by pass only while more than coop_faces of its faces need it; the
-// others go to a list that the CTA's warps then work off with 16 lanes per face, one lane per
-// population (coop_tail).  In FP64 (without the predictor) the list is the whole grid's and a kernel of its
-// own works it off (lane_tail_kernel).
+// others go to a list that is worked off with 16 lanes per face, one lane per population: the whole
+// grid's, by a kernel of its own (lane_tail_kernel), or with the learned predictor the CTA's (coop_tail).
 //
 // Measured (GB300, us a launch; before: the best of the node-by-node tiles, that is 8 x 8 with
 // shared scratch in FP32 and 8 x 8 in FP64, and the 32 x 4 tile that was the default): FP32 quadrants
-// 1024^2 290 (328, default 446), shocked interface 1001 x 253 with minmod 110 (130, 186); FP64
-// quadrants 256^2 965 with the tail kernel (3208; 1310 with the CTA's own tail).  FP32 issues 143 M instructions where the node-by-node tile issued 252 M,
+// 1024^2 280 (328, default 446), shocked interface 1001 x 253 with minmod 93 (130, 186); FP64
+// quadrants 256^2 965 (3208), all with the tail kernel.  FP32 issues 143 M instructions where the node-by-node tile issued 252 M,
 // at 49% of the issue slots with 12 warps per SM: a packed multiply-add with three different
 // register pairs takes four cycles of the register file (two with a repeated operand), the
 // dependent-instruction waits come next (1.6 of 6 cycles), then the loads around the pass.  Four CTAs
@@ -401,20 +400,21 @@ __device__ __forceinline__ void coop_get(const float *o, float *c)
         c[4 * k] = x.x; c[4 * k + 1] = x.y; c[4 * k + 2] = x.z; c[4 * k + 3] = x.w;
     }
 }
-// FP64 without the predictor: the faces that their warps leave go to a list of the whole grid, which
+// Without the predictor the faces that their warps leave go to a list of the whole grid, which
 // lane_tail_kernel works off, instead of to the CTA's own.
 template <typename R, int MODE>
-__host__ __device__ constexpr bool chip_tail() { return sizeof(R) == 8 && MODE == FACE_PLAIN; }
-constexpr int kTailThreads = 128, kTailCtas = 2;
+__host__ __device__ constexpr bool chip_tail() { return MODE == FACE_PLAIN; }
+constexpr int kTailThreads = 128;
+template <typename R> constexpr int tail_ctas() { return sizeof(R) == 8 ? 2 : 4; }
 
-// A warp with at most this many unfinished faces hands them over.  FP32 (64 faces a warp): a pass of
-// the warp costs about as much as one of 12 faces by groups (quadrants 1024^2: 0.302 / 0.290 /
-// 0.289 ms a launch for 6 / 12 / 20; shocked interface 1001 x 253: 0.113 / 0.110 / 0.116).  FP64 (32
-// faces): a pass takes 64 cycles per instruction however few lanes need it, so more go over, and
-// all of them where the whole chip takes them (quadrants 49 x 583 / 64^2 / 256^2, us a launch with
-// the tail: 884 / 495 / 994 for 20, 718 / 375 / 969 for 31; smooth 300^2 2241 and 2266).
+// A warp with at most this many unfinished faces hands them over.  FP32 (64 faces a warp), us a launch with
+// the tail for 12 / 24 / 40 / 63: quadrants 64^2 108 / 57 / 38 / 35, 49 x 583 98 / 63 / 50 / 48, 1024^2 293 / 277 /
+// 280 / 280, interface 1001 x 253 104 / 97 / 93 / 92, smooth 300^2 (two passes everywhere) 53 / 54 / 54 / 62; to
+// the CTA's own list 12 (1024^2 302 / 290 / 289 for 6 / 12 / 20).  FP64 (32 faces): a pass takes 64 cycles per
+// instruction however few lanes need it, so more go over, and all of them where the whole chip takes
+// them (49 x 583 / 64^2 / 256^2: 884 / 495 / 994 for 20, 718 / 375 / 969 for 31; smooth 300^2 2241 and 2266).
 template <typename R, int MODE>
-__host__ __device__ constexpr int coop_faces() { return sizeof(R) == 4 ? 12 : (chip_tail<R, MODE>() ? 31 : 20); }
+__host__ __device__ constexpr int coop_faces() { return sizeof(R) == 4 ? (chip_tail<R, MODE>() ? 40 : 12) : (chip_tail<R, MODE>() ? 31 : 20); }
 // how a face came to the list: to be passed again from its next frame, or after a pass that
 // defined no frame (COOP_BAD), or after a learned prediction that did not hold (COOP_FAIL)
 enum { COOP_BAD = 1, COOP_FAIL = 2, COOP_LEARNED = 4 };
@@ -998,17 +998,19 @@ lane_face_kernel(const Params<2, R> P)
         }
         if constexpr (CHIP) {
             // the face's frames go into its own output planes, then it takes a place in the list
-            const unsigned lists = __ballot_sync(0xffffffffu, flags[0] >= 0);
-            if (lists) {
+#pragma unroll
+            for (int l = 0; l < L; ++l) {
+                const unsigned lists = __ballot_sync(0xffffffffu, flags[l] >= 0);
+                if (!lists) continue;
                 unsigned at = 0;
                 if ((threadIdx.x & 31) == 0) at = atomicAdd(&P.tail->n, __popc(lists));
                 at = __shfl_sync(0xffffffffu, at, 0) + __popc(lists & ((1u << (threadIdx.x & 31)) - 1u));
-                if (flags[0] >= 0) {
-                    const long long f = face(0);
+                if (flags[l] >= 0) {
+                    const long long f = face(l);
                     R *o = (dir == 0 ? P.xf : P.yf) + f;
-                    o[0] = vget(nn, 0); o[nf] = vget(nt, 0); o[2 * nf] = vget(vn, 0); o[3 * nf] = vget(vt, 0);
-                    o[4 * nf] = vget(nT, 0); o[5 * nf] = vget(vT, 0); o[6 * nf] = R(iters[0]);
-                    P.tail_items()[at] = (unsigned long long)f | (unsigned long long)dir << kTailDirShift | (flags[0] & COOP_BAD ? kTailBad : 0ull);
+                    o[0] = vget(nn, l); o[nf] = vget(nt, l); o[2 * nf] = vget(vn, l); o[3 * nf] = vget(vt, l);
+                    o[4 * nf] = vget(nT, l); o[5 * nf] = vget(vT, l); o[6 * nf] = R(iters[l]);
+                    P.tail_items()[at] = (unsigned long long)f | (unsigned long long)dir << kTailDirShift | (flags[l] & COOP_BAD ? kTailBad : 0ull);
                     ++n_act;
                 }
             }
@@ -1070,26 +1072,28 @@ lane_face_kernel(const Params<2, R> P)
     if ((threadIdx.x & 31) == 0 && (n_act || fc.iters)) count_faces(P.diag, fc, n_act);
 }
 
-// Works off the grid's list of unfinished faces (FP64), 16 lanes per face and two faces a warp: the form
+// Works off the grid's list of unfinished faces, 16 lanes per face and two faces a warp: the form
 // of coop_tail, with lane q < 8 holding stencil cell q in registers and velocities relative to the face's
-// own predictor frame.  Faces that take many passes lie together (a shock crosses a few tiles), and
-// FP64 needs a warp on every sub-partition: the list spreads them over the chip.  Measured (GB300, us a
-// launch of face and tail; before: each CTA its own list): quadrants 256^2 965 (1310), 64^2 375 (1007),
-// 49 x 583 720 (1117), interface 401 x 201 1066 (1388), smooth 300^2 2260 (2222).  Two CTAs per SM (three:
-// 5% slower).  Two warps a face, f and g apart, halve the chain of a pass but cost twice the issue:
-// 850 at 49 x 583, 1105 at 256^2.
+// own predictor frame.  Faces that take many passes lie together (a shock crosses a few tiles), so a CTA's
+// own list keeps a few SMs busy while the others are done: the grid's list spreads them over the
+// chip.  Measured (GB300, us a launch of face and tail; before: each CTA its own list): FP64 quadrants 256^2 965
+// (1310), 64^2 365 (1007), 49 x 583 712 (1117), interface 401 x 201 1056 (1388), smooth 300^2 2260 (2222); FP32
+// quadrants 64^2 36 (81), 49 x 583 46 (76), 300^2 55 (107), 1024^2 280 (290), interface 1001 x 253 93 (110).
+// Two CTAs per SM in FP64 (three: 5% slower), four in FP32 (two: 7% slower at 1024^2).  Two warps a face, f and g
+// apart, halve the chain of a pass but cost twice the issue: FP64 850 at 49 x 583, 1105 at 256^2.
 template <typename R>
 __global__ void __launch_bounds__(kTailThreads)
 lane_tail_kernel(const Params<2, R> P)
 {
     using W = typename FrameWords<R>::word;
-    using V = typename VecOf<R>::type;
-    static_assert(VecOf<R>::lanes == 1, "FP64");
     __shared__ __align__(16) R words[kTailThreads / 16][coop_words<R>()];
     const unsigned full = 0xffffffffu;
     const int q = threadIdx.x & 15, lead = threadIdx.x & 16, m = q >> 2, n = q & 3;
     R *cells = words[threadIdx.x >> 4], *mom = cells + 8 * coop_cell<R>();
-    const unsigned int count = P.tail->n;
+    // The first face of a group goes by its place (the groups of different CTAs first), the others by a
+    // ticket: a CTA without a face leaves at once, and a short list costs no atomics.
+    const unsigned int count = P.tail->n, groups = gridDim.x * (kTailThreads / 16);
+    if (blockIdx.x >= count) return;
     const StepC<R> &KC = step_c<R>(*P.clock);
     const NodeTab<R> &tab = node_tab<R>();
     const R Cv = P.Cv_r, tol = P.tol_r, cm = tab.c[m], cn = tab.c[n];
@@ -1104,15 +1108,12 @@ lane_tail_kernel(const Params<2, R> P)
     FaceCount fc{0, 0, 0, 0};
     int dir = 0, iters = 0, fallbacks = 0;
     long long f = 0, nf = 0;
-    LaneCell<V> cell{};
+    LaneCell<R> cell{};
     cell.sym[4] = R(1);   // (a group without a face passes over a cell at rest)
     W ref[2] = {};
     R una = R(0), uta = R(0), dn = R(0), dt = R(0), Tl = R(1), vn = R(0), vt = R(0), vT = R(1);
     bool live = false, have = false, done = false, restarted = false, redo = false, bad = false;
-    auto take = [&]() {
-        unsigned int item = 0;
-        if (q == 0) item = atomicAdd(&P.tail->next, 1u);
-        item = __shfl_sync(lead ? 0xffff0000u : 0x0000ffffu, item, lead);
+    auto take = [&](unsigned int item) {
         live = item < count;
         if (!live) return;
         const unsigned long long it = P.tail_items()[item];
@@ -1134,7 +1135,7 @@ lane_tail_kernel(const Params<2, R> P)
         uta = R(fr_lead(dir ? ref[0] : ref[1]));
         if (q < 8) {
             const int on = q < 4 ? q - 2 : (q < 6 ? -1 : 0), ot = q < 4 ? 0 : ((q & 1) ? 1 : -1);
-            stage_any<R, V>(P, fi + (dir ? ot : on), fj + (dir ? on : ot), KC.cp, KC.ce, ref, 0, cell);
+            stage_any<R, R>(P, fi + (dir ? ot : on), fj + (dir ? on : ot), KC.cp, KC.ce, ref, 0, cell);
             // in face axes
 #pragma unroll
             for (int k = 0; k < 6; ++k) {
@@ -1144,7 +1145,7 @@ lane_tail_kernel(const Params<2, R> P)
             }
         }
     };
-    take();
+    take((threadIdx.x >> 4) * gridDim.x + blockIdx.x);
     for (;;) {
         __syncwarp();
         if (!__any_sync(full, live)) break;
@@ -1259,12 +1260,14 @@ lane_tail_kernel(const Params<2, R> P)
             fc.nonconv += done ? 0 : 1;
             fc.nonphys += have ? 0 : 1;
         }
-        take();
+        unsigned int item = 0;
+        if (q == 0) item = groups + atomicAdd(&P.tail->next, 1u);
+        take(__shfl_sync(half, item, lead));
     }
     if (q == 0 && fc.iters) count_faces(P.diag, fc, 0);
     __syncthreads();
-    if (threadIdx.x == 0 && atomicAdd(&P.tail->ctas, 1u) == gridDim.x - 1) {
-        // every CTA has taken its last ticket: empty the list
+    if (threadIdx.x == 0 && atomicAdd(&P.tail->ctas, 1u) == min(gridDim.x, count) - 1) {
+        // every CTA with a face has taken its last ticket: empty the list
         P.tail->n = 0u;
         P.tail->next = 0u;
         P.tail->ctas = 0u;

@@ -232,12 +232,12 @@ struct Params {
                                       // previous frame; larger moves may reach another fixed point)
     unsigned int *mlp_err;
     int sms;                          // SMs of the device (grid sizes of the grid-stride kernels)
-    TailList *tail;                   // D2Q16 in FP64: the faces left to the tail kernel (items: tail_items())
+    TailList *tail;                   // D2Q16: the faces left to the tail kernel (items: tail_items())
     // host memory: tensor maps of the two state buffers for the TMA-staged face variant (null
     // where the grid does not allow them); read by the launcher, never by a kernel
     const StageMaps *stage_maps;
     // the list's items, one for each face at most, lie in the planes of the learned predictions, which
-    // the steps without the predictor leave alone: 24 (nx + 1) ny bytes or more in FP64, and the
+    // the steps without the predictor leave alone: 24 (nx + 1) ny bytes in xlr, and the
     // faces number (nx + 1) ny + nx (ny + 1) <= 3 (nx + 1) ny
     __device__ unsigned long long *tail_items() const { return reinterpret_cast<unsigned long long *>(xlr); }
     __host__ __device__ long long ncell() const { return nx * ny; }

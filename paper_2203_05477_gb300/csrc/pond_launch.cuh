@@ -24,8 +24,8 @@ struct VList {
 // ---------------------------------------------------------------- face kernel
 
 // D2Q16: the lane kernel (pond_face2.cuh) in tiles that keep whole warps on one direction; us a
-// launch on the 1024^2 quadrants in FP32: 16 x 8 / 3 CTAs per SM 290, 32 x 4 / 3 302, 16 x 8 / 2 318 (the
-// 1001 x 253 interface: 110, 107, 117), against 328-380 for the node-by-node tiles kept below for
+// launch on the 1024^2 quadrants in FP32: 16 x 8 / 3 CTAs per SM 280, 32 x 4 / 3 283, 16 x 8 / 2 302 (the
+// 1001 x 253 interface: 93, 94, 98), against 328-380 for the node-by-node tiles kept below for
 // comparison; FP64 256^2 with the tail kernel: 8 x 4 / 4 961, 8 x 8 / 2 950, 16 x 4 / 2 1330.
 template <int D, typename R>
 struct FaceList;
@@ -38,10 +38,22 @@ template <>
 struct FaceList<2, double> {
     using type = VList<LaneVariant<8, 4, 4>, LaneVariant<8, 8, 2>, LaneVariant<16, 4, 2>>;
 };
+// whether face variant v is the lane kernel (which may leave faces to a tail kernel)
+template <typename L>
+struct LaneAt;
+template <typename... Vs>
+struct LaneAt<VList<Vs...>> {
+    static bool at(int v)
+    {
+        const bool lanes[] = {Vs::LANES...};
+        return lanes[v >= 0 && v < int(sizeof...(Vs)) ? v : 0];
+    }
+};
+
 // The face variant of a D2Q16 FP32 grid before tuning: where every 16 x 8 tile has half an SM to itself, the
-// kernel without the 168-register cap (its tail's passes are the longest chain of a small grid); us a
-// launch capped / uncapped: quadrants 49 x 583 86 / 78, 64^2 94 / 82, 128^2 92 / 79, interface 80 x 229
-// 47 / 44; above the line 300^2 smooth 46 / 48, quadrants 700^2 160 / 169.
+// kernel without the 168-register cap (a pass's chain is what a small grid waits for); us a
+// launch capped / uncapped: quadrants 49 x 583 50 / 46, 64^2 38 / 36, 128^2 41 / 38, interface 80 x 229
+// 40 / 38; above the line 300^2 55 / 56, 700^2 151 / 160.
 inline int face2_default(long long nx, long long ny, int sms) { return ((nx + 16) / 16) * ((ny + 8) / 8) <= 2ll * sms ? 2 : 0; }
 
 template <typename R>

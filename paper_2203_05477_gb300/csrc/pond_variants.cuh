@@ -15,7 +15,7 @@ void launch_face_one(const Params<D, R> &P, cudaStream_t st)
         constexpr int bytes = int(lane_smem_bytes<R, V>());
         cudaFuncSetAttribute(lane_face_kernel<R, MODE, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         lane_face_kernel<R, MODE, V><<<g, lane_threads<R, V>(), bytes, st>>>(P);
-        if constexpr (chip_tail<R, MODE>()) lane_tail_kernel<R><<<kTailCtas * P.sms, kTailThreads, 0, st>>>(P);
+        if constexpr (chip_tail<R, MODE>()) lane_tail_kernel<R><<<tail_ctas<R>() * P.sms, kTailThreads, 0, st>>>(P);
     } else {
     if constexpr (V::TMA) {
         // the tensor maps of the buffer that holds the state now; without them (a grid whose

@@ -46,6 +46,7 @@ __device__ __forceinline__ void vput(Lane2 &a, int l, float x)
     else a.v.x = x;
 }
 __device__ __forceinline__ void vput(double &a, int, double x) { a = x; }
+__device__ __forceinline__ void vput(float &a, int, float x) { a = x; }
 
 __device__ __forceinline__ Lane2 vsqrt(Lane2 a) { return Lane2{make_float2(w_sqrt<float>(a.v.x), w_sqrt<float>(a.v.y))}; }
 __device__ __forceinline__ double vsqrt(double a) { return sqrt(a); }
