@@ -616,7 +616,7 @@ def bench_equilibration(pb, steps=50):
                      "status_ok": d1["status"] == pond.POND_OK}
         s.close()
     out["cost_ratio"] = out["equilibration"]["ms_per_step"] / out["grad"]["ms_per_step"]
-    out["note"] = "%d steps of the workload, FP32, face 32x4 cells / 2 CTA per SM, cell 256 threads for both" % steps
+    out["note"] = "%d steps of the workload, FP32, the default variant of each (Grad: the face kernel by upwind side; equilibration: node by node, 32x4 cells)" % steps
     return out
 
 

@@ -544,7 +544,6 @@ pond_status step_timed_impl(pond_state *s, int64_t n_steps, double *ms)
         if constexpr (D == 2) {
             if (s->learned) {
                 pond::gauge_predict_kernel<R><<<predict_blocks(s), pond::mlp::kThreads, pond::mlp::kInferSmem, s->stream>>>(P);
-                s->launches += 1;
             }
         }
         if (s->scheme == POND_SL || fused_step<D, R>(s, false)) {
@@ -553,15 +552,15 @@ pond_status step_timed_impl(pond_state *s, int64_t n_steps, double *ms)
             else launch_fused<D, R>(s, P);
             CUDA_TRY(cudaEventRecord(ev[2 * k + 1], s->stream));
             CUDA_TRY(cudaEventRecord(ev[2 * k + 2], s->stream));
-            s->launches -= 1;
+            s->launches += 1;
         } else {
             pond::launch_face<D, R>(s->face_v, false, P, s->stream);
             CUDA_TRY(cudaEventRecord(ev[2 * k + 1], s->stream));
             pond::launch_cell_any<D, R>(s->cell_v, P, s->stream);
             CUDA_TRY(cudaEventRecord(ev[2 * k + 2], s->stream));
+            s->launches += step_launches<D, R>(s);
         }
     }
-    s->launches += 2 * n_steps;
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaEventSynchronize(ev.back()));
     for (int64_t k = 0; k < n_steps; ++k) {
@@ -2026,7 +2025,7 @@ pond_status time_grid_step(pond_state *s, const char *saved, const pond::Params<
     CUDA_TRY(cudaEventRecord(ev[0], s->stream));
     for (int k = 0; k < steps; ++k) launch_step<D, R>(s);
     CUDA_TRY(cudaEventRecord(ev[1], s->stream));
-    s->launches += int64_t(steps + 1) * (fused_step<D, R>(s, false) ? 1 : 2);
+    s->launches += int64_t(steps + 1) * (fused_step<D, R>(s, false) ? 1 : step_launches<D, R>(s));
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaEventSynchronize(ev[1]));
     float a = 0.f;
