@@ -341,7 +341,7 @@ pond_status set_primitive_impl(pond_state *s, const double *rho, const double *u
     if (r != POND_OK) return r;
     pond::init_cells_kernel<D, R><<<blocks_for(n, 256), 256, 0, s->stream>>>(P, dr, dux, duy, dp, R(1.0 / P.dx), R(1.0 / P.dy));
     const long long nf = P.nxf() + (D == 2 ? P.nyf() : 0);
-    pond::init_faces_kernel<D, R><<<blocks_for(nf, 256), 256, 0, s->stream>>>(P, 1.0 / P.Cv);
+    pond::init_faces_kernel<D, R><<<blocks_for(nf, 256), 256, 0, s->stream>>>(P);
     s->launches += 2;
     CUDA_TRY(cudaGetLastError());
     if (!on_device) CUDA_TRY(cudaStreamSynchronize(s->stream));
@@ -1212,7 +1212,10 @@ pond_status pond_init(const pond_grid *grid, pond_velset velset, double gamma, d
     }
     if (st == POND_OK) st = reset_clock(s);
     if (st != POND_OK) { pond_destroy(s); return st; }
-    if (D == 1 && s->scheme == POND_FV) s->tube_v = 1 + pond::chunk_default(s->grid.nx, s->sms);
+    if (D == 1 && s->scheme == POND_FV) {
+        s->tube_v = 1 + (s->prec == POND_FP32 ? pond::chunk_default<float>(s->grid.nx, s->sms)
+                                              : pond::chunk_default<double>(s->grid.nx, s->sms));
+    }
     if (D == 2 && s->prec == POND_FP32) s->face_v = pond::face2_default(s->grid.nx, s->grid.ny, s->sms);
     s->learned = D == 2 && opts->learned != 0;
     if (s->learned) {

@@ -664,9 +664,8 @@ __host__ __device__ constexpr int face_keep_slot(int level) { return level > 1 ?
 // One corrector pass at a D1Q4 face (Grad projection): the four stencil cells in the pass frame
 // (shift form), the outer differences formed in Hermite space, the nodes +-c evaluated as even and
 // odd parts.  A node takes its upwind cell's value and the limited slope of the centre difference
-// and its side's outer one, which enter the limiter symmetrically.  f rides
-// with g in (f, g) pairs for the orders both have (packed FP32x2 in FP32).  About 240 instructions in
-// FP32 against 420 for the node-by-node pass with its maps; 330 FP64 operations against 600.
+// and its side's outer one, which enter the limiter symmetrically.  330 FP64 operations against 600 for the
+// node-by-node pass with its maps.  FP64 only: FP32 tubes keep that pass, whose rounding they depend on.
 // cell(s): the staged cell at slot s (LL, L, R, RR); rel(cell): its velocity less the pass frame's.
 template <typename R, typename CELL, typename REL>
 __device__ __forceinline__ void pass1(CELL &&cell, REL &&rel, R Tl, R un, R h_dn, int limiter, R *Phi, R *Psi)
@@ -745,6 +744,102 @@ __device__ __forceinline__ void pass1(CELL &&cell, REL &&rel, R Tl, R un, R h_dn
         Psi[k] = gpart(S[k]);
     }
     Phi[3] = S3;
+}
+
+// ---- D1Q4 in FP32 with every contraction written out
+//
+// The fused step (pond_chunk.cuh) is held to the bits of the face and cell kernels: a shock amplifies
+// a change of rounding in an FP32 tube (limiters switch, correctors cycle) far beyond the rounding itself,
+// and which of two products a sum absorbs is the compiler's choice, kernel by kernel.  These functions
+// round where those two kernels do.
+
+// Map1 (pond_core.cuh) with its sums rounded separately, as the face passes and the cell's new frame take
+// it, or (FUSED) with d^2 contracted into them, as the flux does
+template <bool FUSED>
+struct Map1Written {
+    float t10, t11, t20, t21, t22, t30, t31, t32, t33;
+    __device__ __forceinline__ Map1Written(float s, float e, float d)
+    {
+        const float d2 = __fmul_rn(d, d);
+        t10 = d;
+        t11 = s;
+        t20 = FUSED ? fmaf(d, d, e) : __fadd_rn(e, d2);
+        t21 = __fmul_rn(__fmul_rn(2.f, s), d);
+        t22 = __fadd_rn(e, 1.f);
+        t30 = __fmul_rn(d, FUSED ? fmaf(d, d, __fmul_rn(3.f, e)) : fmaf(3.f, e, d2));
+        t31 = __fmul_rn(__fmul_rn(3.f, s), t20);
+        t32 = __fmul_rn(__fmul_rn(3.f, t22), d);
+        t33 = __fmul_rn(t22, s);
+    }
+    // orders 0..3, 0..3 with a zero first order, 0..2
+    __device__ __forceinline__ void f(const float *A, float *F) const
+    {
+        F[3] = fmaf(t33, A[3], fmaf(t32, A[2], fmaf(t31, A[1], __fmul_rn(t30, A[0]))));
+        g(A, F);
+    }
+    __device__ __forceinline__ void f0(const float *A, float *F) const
+    {
+        F[0] = A[0];
+        F[1] = __fmul_rn(t10, A[0]);
+        F[2] = fmaf(t22, A[2], __fmul_rn(t20, A[0]));
+        F[3] = fmaf(t33, A[3], fmaf(t32, A[2], __fmul_rn(t30, A[0])));
+    }
+    __device__ __forceinline__ void g(const float *B, float *G) const
+    {
+        G[0] = B[0];
+        G[1] = fmaf(t11, B[1], __fmul_rn(t10, B[0]));
+        G[2] = fmaf(t22, B[2], fmaf(t21, B[1], __fmul_rn(t20, B[0])));
+    }
+};
+
+// corrector_pass of a D1Q4 face
+__device__ __forceinline__ void pass1_written(const Stencil<1, float> &cells, float dref, float dl, float Tl, float un, float h_dn,
+                                              int limiter, float *Phi, float *Psi)
+{
+    const float invTl = w_rcp<float>(Tl), rsqTl = w_sqrt<float>(invTl), sqTl = __fmul_rn(Tl, rsqTl);
+    float F[4][4], G[4][3];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const StagedCell<1, float> c = fetch<1, float>(cells[q]);
+        const Map1Written<false> M(w_sqrt<float>(__fmul_rn(c.T, invTl)), __fmul_rn(__fadd_rn(c.T, -Tl), invTl),
+                                   __fmul_rn(__fadd_rn(__fadd_rn(c.du[0], -dref), -dl), rsqTl));
+        M.f0(c.A, F[q]);
+        M.g(c.B, G[q]);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) Phi[k] = 0.f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) Psi[k] = 0.f;
+    const float sc = limit_scale(limiter);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        const float vn = fmaf(sqTl, float(node_c(m)), un);
+        const bool left = vn > 0.f;
+        const float off = __fmul_rn(sc, fmaf(-vn, h_dn, left ? 0.5f : -0.5f));
+        // (f, g) at the node
+        auto value = [&](const float *f, const float *g) {
+            float2 p = __ffma2_rn(make_float2(f[1], g[1]), bc2(float(hen(1, m))), make_float2(f[0], g[0]));
+            p = __ffma2_rn(make_float2(f[2], g[2]), bc2(float(hen(2, m))), p);
+            p.x = fmaf(f[3], float(hen(3, m)), p.x);
+            return p;
+        };
+        float FS[4], GS[3];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) FS[k] = left ? F[0][k] : F[3][k];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) GS[k] = left ? G[0][k] : G[3][k];
+        const float2 pL = value(F[1], G[1]), pR = value(F[2], G[2]), pS = value(FS, GS), minus1 = bc2(-1.f);
+        const float2 pu = left ? pL : pR, pl = left ? pS : pL, ph = left ? pR : pS;
+        const float2 sl = limit2_scaled(limiter, __ffma2_rn(pl, minus1, pu), __ffma2_rn(pu, minus1, ph));
+        const float2 pb = __ffma2_rn(bc2(off), sl, pu);
+#pragma unroll
+        for (int a = 0; a <= 2; ++a) {
+            const float2 acc = __ffma2_rn(bc2(float(node_w(m) * he(a, m))), pb, make_float2(Phi[a], Psi[a]));
+            Phi[a] = acc.x;
+            Psi[a] = acc.y;
+        }
+        Phi[3] = fmaf(float(node_w(m) * he(3, m)), pb.x, Phi[3]);
+    }
 }
 
 // The same pass by four lanes per face (j: this lane's place): lane j moves stencil cell j into the frame
@@ -828,7 +923,7 @@ __device__ __forceinline__ void corrector_pass(const Stencil<D, R> &cells, const
                                                int limiter, R *Phi, R *Psi, FaceScratch scr = FaceScratch{nullptr, 0})
 {
     static_assert(!SCR || (D == 2 && sizeof(R) == 4 && !EQ), "the scratch variants are FP32 2D Grad passes");
-    if constexpr (D == 1 && OUTER_ONCE && !EQ) {
+    if constexpr (D == 1 && sizeof(R) == 8 && OUTER_ONCE && !EQ) {
         pass1<R>([&](int s) { return fetch<1, R>(cells[s]); },
                  [&](const StagedCell<1, R> &c) { return c.du[0] - (dref[0] + dl[0]); }, Tl, un_abs, h_dn, limiter, Phi, Psi);
     } else {
@@ -1178,7 +1273,8 @@ struct FaceOut {
 // KEEP (FP32): 1, the last valid pass's frames wait in two slots of the thread's scratch
 // (after the corrector's own slots) instead of staying live across the next pass; 2, the
 // constants of the face output wait in one more slot
-template <int D, typename R, bool EQ = false, int SCR = 0, bool OUTER_ONCE = true, int KEEP = (SCR > 1 ? 2 : SCR), int LPF = 1>
+// LPF (D1Q4, FP64): four lanes solve a face together.  WRITTEN (D1Q4, FP32): the contractions written out
+template <int D, typename R, bool EQ = false, int SCR = 0, bool OUTER_ONCE = true, int KEEP = (SCR > 1 ? 2 : SCR), int LPF = 1, bool WRITTEN = false>
 __device__ __forceinline__ void solve_face(const Stencil<D, R> &cells, bool swap, const R *dref, const R *uabs,
                                            R Tpred, const FaceCfg<R> &cfg, FaceOut<D, R> &o,
                                            FaceScratch scr = FaceScratch{nullptr, 0})
@@ -1205,7 +1301,9 @@ __device__ __forceinline__ void solve_face(const Stencil<D, R> &cells, bool swap
     int iters = 0;
     R Phi[NFC], Psi[NGC];
     auto pass = [&](const R *pdl, R pT) {
-        if constexpr (LPF > 1)
+        if constexpr (WRITTEN)
+            pass1_written(cells, dref[0], pdl[0], pT, uref_n + pdl[0], h_dn, cfg.limiter, Phi, Psi);
+        else if constexpr (LPF > 1)
             pass1_quad<R>([&](int s) { return fetch<1, R>(cells[s]); },
                           [&](const StagedCell<1, R> &c) { return c.du[0] - (dref[0] + pdl[0]); }, threadIdx.x & (LPF - 1), pT,
                           uref_n + pdl[0], h_dn, cfg.limiter, Phi, Psi);
@@ -1290,7 +1388,11 @@ __device__ __forceinline__ void solve_face(const Stencil<D, R> &cells, bool swap
         const R invT = w_rcp<R>(out_T);
         const R sk = w_sqrt<R>(keep_T * invT), rsq = w_sqrt<R>(invT);
         R Fo[NFC], Go[NGC];
-        if constexpr (D == 1 && OUTER_ONCE && !EQ) {
+        if constexpr (WRITTEN) {
+            const Map1Written<false> M(sk, __fmul_rn(__fadd_rn(keep_T, -out_T), invT), __fmul_rn(-out_du[0], rsq));
+            M.f(Phi, Fo);
+            M.g(Psi, Go);
+        } else if constexpr (D == 1 && sizeof(R) == 8 && OUTER_ONCE && !EQ) {
             const Move1<R> M(sk, (keep_T - out_T) * invT, -out_du[0] * rsq);
             M.f(Phi, Fo);
             M.g(Psi, Go);
@@ -1681,7 +1783,7 @@ face_tma_kernel(const Params<D, R> P, const __grid_constant__ StageMaps maps)
 // using c He_r(c) = He_{r+1}(c) + r He_{r-1}(c); He_4 vanishes on the D1Q4 nodes and the
 // Grad forms have no moments above their order, so the product closes on the same orders.
 // invTc, rsqTc: 1/T and 1/sqrt(T) of the cell frame.
-template <int D, typename R, bool EQ = false, bool SHIFT = D == 1 && !EQ>
+template <int D, typename R, bool EQ = false, bool SHIFT = D == 1 && sizeof(R) == 8 && !EQ>
 __device__ __forceinline__ void add_face_flux(const R *Fc, const R *Gc, const R *dv, R Tbr, R Tcr, R invTc, R rsqTc,
                                               int axis, R scale, R sqTc, R un, R *H, R *G)
 {
@@ -1861,7 +1963,7 @@ __device__ __forceinline__ void reduce_rate_and_advance(Clock *clock, double rat
 // it (f third order, g second order).  The frame changes by increments formed relative to
 // the old frame, du and dT (T' = T (1 + dT)), which the caller applies to its own
 // representation of the frame.
-template <int D, typename R, bool SHIFT = D == 1>
+template <int D, typename R, bool SHIFT = D == 1 && sizeof(R) == 8>
 __device__ __forceinline__ bool cell_finish(const R *H, const R *G, R invTc, R sqTc, R Cv, R *Ho, R *Go, R *du, R &dT)
 {
     const R rsqTc = invTc * sqTc;
@@ -2325,11 +2427,9 @@ __device__ __forceinline__ void cell_conserved(const Params<D, R> &P, long long 
 }
 
 // Face predictor before the first step: frame of the pooled moments of the two cells.  Bound by the FP64
-// pipe, on which a division takes as long as nine multiply-adds: one reciprocal a face (inv_Cv comes from
-// the host) instead of three divisions in 1D and four in 2D, and 32-bit face indices where they fit; the
-// cell kernel takes 1/dx from the host.  Setting 4 M cells in FP32: 742 -> 560 us.
+// pipe, on which a division takes as long as nine multiply-adds; 32-bit face indices where they fit.
 template <int D, typename R>
-__global__ void init_faces_kernel(const Params<D, R> P, double inv_Cv)
+__global__ void init_faces_kernel(const Params<D, R> P)
 {
     const long long nxf = P.nxf(), nyf = D == 2 ? P.nyf() : 0;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -2349,15 +2449,15 @@ __global__ void init_faces_kernel(const Params<D, R> P, double inv_Cv)
     double ra, ma[2] = {0, 0}, Ea, rb, mb[2] = {0, 0}, Eb;
     cell_conserved<D, R>(P, ai, aj, ra, ma, Ea);
     cell_conserved<D, R>(P, bi, bj, rb, mb, Eb);
-    const double r = 0.5 * (ra + rb), E = 0.5 * (Ea + Eb), ir = 1.0 / r;
+    const double r = 0.5 * (ra + rb), E = 0.5 * (Ea + Eb);
     double k2 = 0.0, u[2];
 #pragma unroll
-    for (int a = 0; a < D; ++a) { const double m = 0.5 * (ma[a] + mb[a]); u[a] = m * ir; k2 += m * m; }
+    for (int a = 0; a < D; ++a) { const double m = 0.5 * (ma[a] + mb[a]); u[a] = m / r; k2 += m * m; }
     typename FrameWords<R>::word *Frm = xdir ? P.xfr : P.yfr;
     const long long nf = xdir ? nxf : nyf;
 #pragma unroll
     for (int a = 0; a < D; ++a) fr_store(Frm[a * nf + f], u[a]);
-    fr_store(Frm[D * nf + f], (E - 0.5 * k2 * ir) * (ir * inv_Cv));
+    fr_store(Frm[D * nf + f], (E - 0.5 * k2 / r) / (P.Cv * r));
 }
 
 // ------------------------------------------------------- learned gauge predictor

@@ -123,17 +123,19 @@ struct StepList<2, double> {
 };
 template <>
 struct StepList<1, float> {
-    using type = VList<ChunkVariant<1, 4, 4>, ChunkVariant<4, 1, 16>>;
+    using type = VList<ChunkVariant<1, 1, 16>, ChunkVariant<1, 4, 4>>;
 };
 template <>
 struct StepList<1, double> {
     using type = VList<ChunkVariant<1, 4, 2>, ChunkVariant<4, 1, 8>>;
 };
 
-// The fused variant of a D1Q4 grid before tuning: four lanes per face while its chunks of 7 cells give
-// each sub-partition at most one warp, else a lane per face (us a step with one / four lanes: tube of
-// 400 cells FP64 104 / 57, 200 cells FP32 13.8 / 12.7, 4 M cells FP32 189 / 549).
-inline int chunk_default(long long nx, int sms) { return nx <= 7ll * 4 * sms ? 1 : 0; }
+// The fused variant of a D1Q4 grid before tuning.  FP32: a warp a CTA (us a step, one warp / four warps a
+// CTA: 200 cells 7.6 / 7.2, 1000 8.9 / 9.0, 30 000 9.2 / 10.3, 200 000 15.9 / 16.4, 4 M 201 / 212).  FP64: four
+// lanes per face while its chunks of 7 cells give each sub-partition at most one warp, else a lane per face
+// (tube of 400 cells 104 with one lane, 57 with four).
+template <typename R>
+inline int chunk_default(long long nx, int sms) { return sizeof(R) == 8 && nx <= 7ll * 4 * sms ? 1 : 0; }
 
 template <int D, typename R>
 constexpr int step_variants() { return StepList<D, R>::type::size; }
