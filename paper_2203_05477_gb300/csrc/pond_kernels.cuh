@@ -842,13 +842,27 @@ __device__ __forceinline__ void pass1_written(const Stencil<1, float> &cells, fl
     }
 }
 
-// The same pass by four lanes per face (j: this lane's place): lane j moves stencil cell j into the frame
+// The sum of a product over the four lanes of a quad, the same bits in each: the products are rounded before
+// the first exchange.  (Contracted into the first addition, each lane would round the other one's product and
+// keep its own exact.)
+__device__ __forceinline__ double quad_sum(unsigned quad, double a, double b)
+{
+    double v = __dmul_rn(a, b);
+    v += __shfl_xor_sync(quad, v, 1);
+    return v + __shfl_xor_sync(quad, v, 2);
+}
+
+// pass1 by four lanes per face (j: this lane's place): lane j moves stencil cell j into the frame
 // and evaluates node j, and the moments are summed across the four.  A quarter of the work is
 // serial per lane: 130 FP64 operations a pass against 330 (an FP64 instruction takes 64 cycles
-// whatever the number of lanes), for grids too small to fill the chip with a lane per face.
-template <typename R, typename CELL, typename REL>
-__device__ __forceinline__ void pass1_quad(CELL &&cell, REL &&rel, int j, R Tl, R un, R h_dn, int limiter, R *Phi, R *Psi)
+// whatever the number of lanes), for grids too small to fill the chip with a lane per face.  Every lane
+// goes on or stops by its own copy of the moments (solve_face) and the next pass exchanges among all four, so
+// the copies must be equal to the last bit (quad_sum).
+template <typename CELL, typename REL>
+__device__ __forceinline__ void pass1_quad(CELL &&cell, REL &&rel, int j, double Tl, double un, double h_dn, int limiter, double *Phi,
+                                           double *Psi)
 {
+    using R = double;
     const unsigned quad = 0xfu << (threadIdx.x & 28);
     const int first = threadIdx.x & 28;
     const R invTl = w_rcp<R>(Tl), rsqTl = w_sqrt<R>(invTl), sqTl = Tl * rsqTl;
@@ -892,18 +906,9 @@ __device__ __forceinline__ void pass1_quad(CELL &&cell, REL &&rel, int j, R Tl, 
         gu = vfma(R(2) * off, vanleer_half(gu - gl, gh - gu), gu);
     }
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        R v = tab.whe[j][a] * fu;
-        v += __shfl_xor_sync(quad, v, 1);
-        v += __shfl_xor_sync(quad, v, 2);
-        Phi[a] = v;
-        if (a < 3) {
-            R w = tab.whe[j][a] * gu;
-            w += __shfl_xor_sync(quad, w, 1);
-            w += __shfl_xor_sync(quad, w, 2);
-            Psi[a] = w;
-        }
-    }
+    for (int a = 0; a < 4; ++a) Phi[a] = quad_sum(quad, tab.whe[j][a], fu);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) Psi[a] = quad_sum(quad, tab.whe[j][a], gu);
 }
 
 // One corrector pass at a face (Sec. III.B.3) in frame (dl, Tl) (velocity relative to the
@@ -1304,9 +1309,9 @@ __device__ __forceinline__ void solve_face(const Stencil<D, R> &cells, bool swap
         if constexpr (WRITTEN)
             pass1_written(cells, dref[0], pdl[0], pT, uref_n + pdl[0], h_dn, cfg.limiter, Phi, Psi);
         else if constexpr (LPF > 1)
-            pass1_quad<R>([&](int s) { return fetch<1, R>(cells[s]); },
-                          [&](const StagedCell<1, R> &c) { return c.du[0] - (dref[0] + pdl[0]); }, threadIdx.x & (LPF - 1), pT,
-                          uref_n + pdl[0], h_dn, cfg.limiter, Phi, Psi);
+            pass1_quad([&](int s) { return fetch<1, R>(cells[s]); },
+                       [&](const StagedCell<1, R> &c) { return c.du[0] - (dref[0] + pdl[0]); }, threadIdx.x & (LPF - 1), pT,
+                       uref_n + pdl[0], h_dn, cfg.limiter, Phi, Psi);
         else
             corrector_pass<D, R, EQ, SCR, OUTER_ONCE>(cells, dref, pdl, pT, uref_n + pdl[0], D == 2 ? uref_t + pdl[D - 1] : R(0),
                                                       h_dn, h_dt, cfg.limiter, Phi, Psi, scr);

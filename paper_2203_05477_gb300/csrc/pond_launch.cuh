@@ -133,7 +133,8 @@ struct StepList<1, double> {
 // The fused variant of a D1Q4 grid before tuning.  FP32: a warp a CTA (us a step, one warp / four warps a
 // CTA: 200 cells 7.6 / 7.2, 1000 8.9 / 9.0, 30 000 9.2 / 10.3, 200 000 15.9 / 16.4, 4 M 201 / 212).  FP64: four
 // lanes per face while its chunks of 7 cells give each sub-partition at most one warp, else a lane per face
-// (tube of 400 cells 104 with one lane, 57 with four).
+// (one / four lanes: 200 cells 70 / 39, 400 107 / 58, 1000 115 / 61, 4000 106 / 57; beyond the line, which is on
+// the safe side of the crossing: 5000 105 / 57, 8000 98 / 60, 12 000 98 / 69, 20 000 96 / 114).
 template <typename R>
 inline int chunk_default(long long nx, int sms) { return sizeof(R) == 8 && nx <= 7ll * 4 * sms ? 1 : 0; }
 
