@@ -278,7 +278,9 @@ sl2_kernel(const Params<2, R> P)
             pf[k] = limited(pf[k], af[k], bf[k], f1[k], f2[k]);
             pg[k] = limited(pg[k], ag[k], bg[k], g1[k], g2[k]);
         }
-        // moments along y, then of all lanes' c_m
+        // Moments along y, then of all lanes' c_m.  Each lane stops by its own copy of them and moves its
+        // stencil nodes into its own frame, so the copies must agree to the last bit: the product is rounded
+        // before the exchange (contracted into the sum, each lane would round the other one's).
         R S[4] = {R(0), R(0), R(0), R(0)}, SG[3] = {R(0), R(0), R(0)};
 #pragma unroll
         for (int hi = 0; hi < 2; ++hi) {
@@ -288,7 +290,8 @@ sl2_kernel(const Params<2, R> P)
             S[0] = vfma(v0, s, S[0]); S[1] = vfma(v1, d, S[1]); S[2] = vfma(v2, s, S[2]); S[3] = vfma(v3, d, S[3]);
             SG[0] = vfma(v0, sg, SG[0]); SG[1] = vfma(v1, dg, SG[1]); SG[2] = vfma(v2, sg, SG[2]);
         }
-        auto over_lanes = [&](R v) {
+        auto over_lanes = [&](R a, R b) {
+            R v = vmul_rn(a, b);
             v += __shfl_xor_sync(0xffffffffu, v, 8);
             return v + __shfl_xor_sync(0xffffffffu, v, 16);
         };
@@ -296,9 +299,9 @@ sl2_kernel(const Params<2, R> P)
         for (int r = 0; r <= 3; ++r) {
             const R w = tab.whe[m][r];
 #pragma unroll
-            for (int s = 0; r + s <= 3; ++s) Phi[hidx(r, s)] += over_lanes(w * S[s]);
+            for (int s = 0; r + s <= 3; ++s) Phi[hidx(r, s)] += over_lanes(w, S[s]);
 #pragma unroll
-            for (int s = 0; r + s <= 2; ++s) Psi[hidx(r, s)] += over_lanes(w * SG[s]);
+            for (int s = 0; r + s <= 2; ++s) Psi[hidx(r, s)] += over_lanes(w, SG[s]);
         }
     };
     bool running = active;

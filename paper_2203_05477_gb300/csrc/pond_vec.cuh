@@ -37,6 +37,10 @@ __device__ __forceinline__ Lane2 vfma(Lane2 a, Lane2 b, Lane2 c) { return Lane2{
 __device__ __forceinline__ double vfma(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
 
+// a product that no sum may absorb
+__device__ __forceinline__ double vmul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float vmul_rn(float a, float b) { return __fmul_rn(a, b); }
+
 // the lane l (0 or 1) of a value
 __device__ __forceinline__ float vget(const Lane2 &a, int l) { return l ? a.v.y : a.v.x; }
 __device__ __forceinline__ double vget(const double &a, int) { return a; }
