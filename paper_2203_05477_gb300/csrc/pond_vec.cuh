@@ -4,8 +4,9 @@
 // FP32 kernels carry two faces per thread, one in each lane of the FP32x2 instructions of
 // sm_100 and later (Lane2): both faces run the same operations on their own data, so every
 // multiply-add serves two and no operand has to be broadcast or paired up.  FP64 kernels
-// carry one face per thread (double).  The code between the two is the same template; every
-// contraction is written out (vfma), so both round where they say they do.
+// carry one face per thread (double).  The code between the two is the same template.  Lane2 operations
+// round where they say (each is one instruction); in scalar code of the same templates, in FP64 and in the FP32
+// tails, the compiler may contract a product that is not written as vfma into a sum.
 #pragma once
 
 #include "pond_core.cuh"
