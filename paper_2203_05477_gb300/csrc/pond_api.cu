@@ -412,7 +412,8 @@ void launch_sl(pond_state *s, pond::Params<D, R> &P)
         pond::sl_kernel<R, kSlThreads><<<blocks_for(P.nx, kSlThreads), kSlThreads, 0, s->stream>>>(P);
     } else {
         using T = Sl2<R>;
-        const dim3 g(unsigned((P.nx + T::TX - 1) / T::TX), unsigned((P.ny + T::TY - 1) / T::TY));
+        const long long rows = (P.ny + T::TY - 1) / T::TY, layers = T::LAYERS ? (rows + 65534) / 65535 : 1;
+        const dim3 g(unsigned((P.nx + T::TX - 1) / T::TX), unsigned((rows + layers - 1) / layers), unsigned(layers));
         pond::sl2_kernel<R, T><<<g, T::THREADS, T::scratch, s->stream>>>(P);
     }
     std::swap(P.sf, P.xf);

@@ -76,6 +76,7 @@ struct Sl2Scratch {
 template <typename R, int TX_, int TY_, int MINB_>
 struct Sl2Tile {
     static constexpr int TX = TX_, TY = TY_, MINB = MINB_, THREADS = 4 * TX * TY;
+    static constexpr bool LAYERS = TY < 8;   // tile rows past 65 535 along gridDim.z
     static constexpr size_t scratch = size_t(TX) * TY * Sl2Scratch<R>::NODE * sizeof(R);
     static_assert(TX == 8, "a warp takes eight nodes of a row");
 };
@@ -120,7 +121,10 @@ sl2_kernel(const Params<2, R> P)
     if (!(K.dt > 0.0)) return;
     const StepC<R> &KC = step_c<R>(K);
     const long long n = P.ncell();
-    const long long i0 = (long long)blockIdx.x * TX, j0 = (long long)blockIdx.y * TY;
+    // gridDim.y ends at 65 535 tile rows; FP64 tiles, of two nodes a row, go on along z, a row past the grid updating
+    // nothing (in FP32, whose tiles are 8 high, the two more indices would spill: 500^2 163 -> 173 us a step)
+    const long long i0 = (long long)blockIdx.x * TX;
+    const long long j0 = (V::LAYERS ? (long long)blockIdx.z * gridDim.y + blockIdx.y : (long long)blockIdx.y) * TY;
     W ut[2];   // every thread reads it (the same words), so the staging needs no barrier before it
     cell_velocity<2, R>(P, i0, j0, ut);
     if (threadIdx.x < 2) utile[threadIdx.x] = threadIdx.x ? ut[1] : ut[0];
