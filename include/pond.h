@@ -347,7 +347,10 @@ const char *pond_variant_name(const pond_state *s, int i);
    face and cell kernels; k > 0: fused step variant k - 1, used for the plain steps -- the
    learned predictor, pair collection and the equilibration ablation run the face and cell
    kernels); for a D3Q64 grid face and cell (`tube` must be 0); for a batch tube (the others
-   are ignored).  Errors: INVALID_ARG for an index out of range. */
+   are ignored).  What an index stands for can change with the library: pond_variant_name says.  A D2Q16
+   grid takes face indices 0 to 13 (FP32) or 0 to 3 (FP64), as many as its longest list had; one past
+   the present list selects the variant that the grid starts on.  Errors: INVALID_ARG for an
+   index out of range. */
 pond_status pond_set_variants(pond_state *s, int face, int cell, int tube);
 
 /* Waits for the stream and reports the device diagnostics.  Returns

@@ -197,6 +197,12 @@ bool encode_stage_maps(pond_state *s, long long nx, long long ny, const R *sf0, 
     return true;
 }
 
+// the face variant that a grid starts on
+int default_face(const pond_state *s)
+{
+    return s->D == 2 && s->prec == POND_FP32 ? pond::face2_default(s->grid.nx, s->grid.ny, s->sms) : 0;
+}
+
 template <int D, typename R>
 pond_status setup(pond_state *s)
 {
@@ -1217,7 +1223,7 @@ pond_status pond_init(const pond_grid *grid, pond_velset velset, double gamma, d
         s->tube_v = 1 + (s->prec == POND_FP32 ? pond::chunk_default<float>(s->grid.nx, s->sms)
                                               : pond::chunk_default<double>(s->grid.nx, s->sms));
     }
-    if (D == 2 && s->prec == POND_FP32) s->face_v = pond::face2_default(s->grid.nx, s->grid.ny, s->sms);
+    s->face_v = default_face(s);
     s->learned = D == 2 && opts->learned != 0;
     if (s->learned) {
         if (s->prec == POND_FP32) params_of<2, float>(s).use_learned = 1;
@@ -2267,7 +2273,9 @@ pond_status pond_set_variants(pond_state *s, int face, int cell, int tube)
         s->cell_v = cell;
         s->tube_v = 0;
     } else {
-        const int nf = grid_face_variants(s);
+        // D2Q16: the list held kFaceIndices once; an index past its present end stands for the starting variant
+        const int nf = grid_face_variants(s), most = s->D == 2 ? pond::kFaceIndices[s->prec == POND_FP32 ? 0 : 1] : nf;
+        if (face >= nf && face < most) face = default_face(s);
         if (face < 0 || face >= nf || cell < 0 || cell >= pond::kCellVariants)
             return fail(POND_ERR_INVALID_ARG, "face/cell variant (%d, %d) out of range", face, cell);
         if (tube < 0 || tube >= grid_step_variants(s) || (tube > 0 && s->scheme != POND_FV))

@@ -38,6 +38,8 @@ template <>
 struct FaceList<2, double> {
     using type = VList<LaneVariant<8, 4, 4>, LaneVariant<8, 8, 2>, LaneVariant<16, 4, 2>>;
 };
+// D2Q16 face indices that pond_set_variants takes, FP32 and FP64: as many as the longest lists had
+constexpr int kFaceIndices[2] = {14, 4};
 // whether face variant v is the lane kernel (which may leave faces to a tail kernel)
 template <typename L>
 struct LaneAt;
