@@ -78,6 +78,7 @@ tube_kernel(const TubeParams<R> P, int steps, int cur0)
 {
     constexpr int NW = THREADS / 32;
     constexpr int kStage = kTubeChunk + 4;
+    constexpr bool AHEAD = THREADS * MINB <= 512;   // 128 registers a thread or more
     using CellW = typename FrameWords<R>::word;
     __shared__ StagedCell<1, R> tile[NW][kStage];
     __shared__ R faceF[NW][kTubeChunk + 1][4];
@@ -155,22 +156,27 @@ tube_kernel(const TubeParams<R> P, int steps, int cur0)
         const R Cvh = CvR - R(0.5);
         const R *sf = P.sf[cur] + c_off, *sg = P.sg[cur] + c_off;
         const CellW *sfr = P.sfr[cur] + c_off;
-        // A chunk's loads are issued before the previous chunk is solved.  Lane l stages cell c0 - 2 + l
-        // (zero-gradient ends) and keeps its state for the update below; lanes 0 and 1 also stage the
-        // right halo c0 + 30, c0 + 31.
+        // A chunk's loads are issued before the previous chunk is solved, but at 80 registers (AHEAD false), where they
+        // spill 272 B (us a step over 1000 steps, 256 threads / 3 CTAs: 176 ahead, 165 not; 256 / 2: 167 ahead,
+        // 189 not; 128 / 4: 181 ahead, 240 not).  Lane l stages cell c0 - 2 + l (zero-gradient ends) and keeps its
+        // state for the update below; lanes 0 and 1 also stage the right halo c0 + 30, c0 + 31.
         R rho{}, a2{}, a3{}, b0{}, b1{}, b2{}, fT{};
         CellW uc{}, Tc{};
         typename TubeParams<R>::FaceW fu{};
         R h[6]{}, hT{};
         CellW hu{};
+        auto load_face = [&](int c0) {
+            const unsigned int k = min(c0 + lane, L);
+            fu = fu_in[k];
+            fT = R(fT_in[k]);
+        };
         auto load = [&](int chunk) {
             const int c0 = chunk * kTubeChunk;
-            const unsigned int c = min(max(c0 - 2 + lane, 0), L - 1), k = min(c0 + lane, L);
+            const unsigned int c = min(max(c0 - 2 + lane, 0), L - 1);
             rho = sf[c]; a2 = (sf + n)[c]; a3 = (sf + 2 * n)[c];
             b0 = sg[c]; b1 = (sg + n)[c]; b2 = (sg + 2 * n)[c];
             uc = sfr[c]; Tc = (sfr + n)[c];
-            fu = fu_in[k];
-            fT = R(fT_in[k]);
+            if (AHEAD) load_face(c0);
             if (lane < 2) {
                 const unsigned int q = min(c0 + kTubeChunk + lane, L - 1);
                 h[0] = sf[q]; h[1] = (sf + n)[q]; h[2] = (sf + 2 * n)[q];
@@ -194,8 +200,9 @@ tube_kernel(const TubeParams<R> P, int steps, int cur0)
         // a warp held up by a chunk whose faces need many corrector passes does fewer chunks
         // (the state and predictors are double-buffered, so the order does not matter)
         int ci = warp;
-        if (ci * kTubeChunk < L) load(ci);
+        if (AHEAD && ci * kTubeChunk < L) load(ci);
         while (ci * kTubeChunk < L) {
+            if (!AHEAD) load(ci);
             const int c0 = ci * kTubeChunk;
             const int nc = min(kTubeChunk, L - c0);
             // reference velocity of the chunk: its first cell's frame velocity
@@ -211,13 +218,17 @@ tube_kernel(const TubeParams<R> P, int steps, int cur0)
             raw[warp][0][lane] = rho; raw[warp][1][lane] = a2; raw[warp][2][lane] = a3;
             raw[warp][3][lane] = b0; raw[warp][4][lane] = b1; raw[warp][5][lane] = b2;
             raww[warp][0][lane] = uc; raww[warp][1][lane] = Tc;
+            if (!AHEAD) load_face(c0);
             const typename TubeParams<R>::FaceW fu_c = fu;
             const R fT_c = fT;
             int nxt_c = 0;
-            if (lane == 0) nxt_c = atomicAdd(&next_chunk, 1);
-            nxt_c = __shfl_sync(0xffffffffu, nxt_c, 0);
+            auto claim = [&] {
+                if (lane == 0) nxt_c = atomicAdd(&next_chunk, 1);
+                nxt_c = __shfl_sync(0xffffffffu, nxt_c, 0);
+            };
+            if (AHEAD) claim();
             __syncwarp();
-            if (nxt_c * kTubeChunk < L) load(nxt_c);
+            if (AHEAD && nxt_c * kTubeChunk < L) load(nxt_c);
             // faces c0 .. c0+nc: face k lies between cells k-1 and k; the last one is also the
             // next chunk's first face, which that chunk owns (except at the tube's end)
             if (lane <= nc) {
@@ -322,6 +333,7 @@ tube_kernel(const TubeParams<R> P, int steps, int cur0)
                 }
             }
             __syncwarp();   // the chunk's shared records are read before the next chunk restages them
+            if (!AHEAD) claim();
             ci = nxt_c;
         }
         // the tube's next time step from its CFL maximum (Sec. IV)
