@@ -21,8 +21,12 @@
 //     lane, spread over the whole chip (face3_tail_kernel): such a face is a chain of up to 15
 //     passes, and the few tiles at a shock hold most of them.
 //
+// Reciprocals, square roots and quotients are the IEEE ones in FP32 too: the hardware's approximations gain 3.5%
+// (64^3 0.71 ms) and cost accuracy, over 30 explosions and smooth flows an error against 64 bits 1.01 times that of the
+// node-by-node kernel, where it is 0.93 times with these.
+//
 // Measured (GB300, ms a step's faces, before: the node-by-node kernel this one replaces): FP32 explosion
-// 64^3 0.71 (1.76), FP64 explosion 25 x 23 x 21 2.2 (15.3).  FP32 issues 52% of the slots with 12 warps
+// 64^3 0.74 (1.76), FP64 explosion 25 x 23 x 21 2.2 (15.3).  FP32 issues 52% of the slots with 12 warps
 // per SM (168 registers, no spills), the rest are dependent-instruction waits and the barrier;
 // FP64 is bound by its pipe (57% busy in the first pass, 65% in the tail).
 #pragma once
@@ -87,7 +91,7 @@ struct Move3 {
     R s, e, d[3], s2, s3;
     __device__ __forceinline__ Move3(R Tc, const R *u, R Tl, R invTl, R rsqTl, const R *l)
     {
-        s = vsqrt(Tc * invTl);
+        s = sqrt(Tc * invTl);
         e = (Tc - Tl) * invTl;
 #pragma unroll
         for (int a = 0; a < 3; ++a) d[a] = (u[a] - l[a]) * rsqTl;
@@ -340,7 +344,7 @@ __device__ __forceinline__ void pass3(const R *base, const FaceAxes3<R> &ax, con
                                       const R *h, int limiter, const SCR &scr, R *Phi, R *Psi)
 {
     const NodeTab<R> &tab = node_tab<R>();
-    const R invTl = vrcp(Tl), rsqTl = vsqrt(invTl), sqTl = Tl * rsqTl;
+    const R invTl = R(1) / Tl, rsqTl = sqrt(invTl), sqTl = Tl * rsqTl;
     // departure offsets with the limiter's factor (2 for van Leer, 1 for minmod)
     const R sc = limiter == 1 ? R(1) : R(2);
 #pragma unroll
@@ -459,15 +463,14 @@ __device__ __forceinline__ bool moments_frame3(const R *p, const R *g, R Tl, R s
 {
     // p: 000, 100, 010, 001, 200, 020, 002
     rho = p[0];
-    const R ir = vrcp(rho);
     R k2 = R(0);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        du[a] = sq * p[1 + a] * ir;
+        du[a] = sq * p[1 + a] / rho;
         k2 = vfma(du[a], du[a], k2);
     }
     const R tr = vfma(R(3), rho, p[4] + p[5] + p[6]);
-    T1 = (vfma(R(0.5) * Tl, tr, g[0]) - R(0.5) * rho * k2) * vrcp(Cv * rho);
+    T1 = (vfma(R(0.5) * Tl, tr, g[0]) - R(0.5) * rho * k2) / (Cv * rho);
     return T1 > R(0) && isfinite(T1) && isfinite(rho) && isfinite(du[0]) && isfinite(du[1]) && isfinite(du[2]);
 }
 
@@ -476,8 +479,8 @@ template <typename R>
 __device__ __forceinline__ void face_populations3(const R *Phi, const R *Psi, R Tl, R rho, const R *du, R T1, R wb, R we,
                                                   R Cvh, R *Fo, R *Go)
 {
-    const R invT = vrcp(T1), zero[3] = {R(0), R(0), R(0)}, u[3] = {-du[0], -du[1], -du[2]};
-    const Move3<R> M(Tl, u, T1, invT, vsqrt(invT), zero);
+    const R invT = R(1) / T1, zero[3] = {R(0), R(0), R(0)}, u[3] = {-du[0], -du[1], -du[2]};
+    const Move3<R> M(Tl, u, T1, invT, sqrt(invT), zero);
     M.f_full(Phi, Fo);
     const R B1[3] = {Psi[1], Psi[2], Psi[3]}, B2[3] = {Psi[4], Psi[7], Psi[9]}, B11[3] = {Psi[8], Psi[6], Psi[5]};
     M.g(Psi[0], B1, B2, B11, Go);
@@ -652,7 +655,7 @@ face3_tail_kernel(const Params3<R> P)
                 }
             }
             // ---- the pass
-            const R invTl = vrcp(Tl), rsqTl = vsqrt(invTl), sqTl = Tl * rsqTl, sq = vsqrt(Tl);
+            const R invTl = R(1) / Tl, rsqTl = sqrt(invTl), sqTl = Tl * rsqTl, sq = sqrt(Tl);
             __syncwarp();
             if (q < 12) {
                 R F[kNF3], G[kNG3];
@@ -856,7 +859,7 @@ face3_kernel(const Params3<R> P)
     for (;;) {
         const R l[3] = {b[0] + d[0], b[1] + d[1], b[2] + d[2]}, ua[3] = {ba[0] + d[0], ba[1] + d[1], ba[2] + d[2]};
         pass3<R, Scr>(base, ax, st, l, Tl, ua, h, P.limiter, scr, Phi, Psi);
-        const R sq = vsqrt(Tl), p[7] = {Phi[0], Phi[1], Phi[2], Phi[3], Phi[4], Phi[7], Phi[9]};
+        const R sq = sqrt(Tl), p[7] = {Phi[0], Phi[1], Phi[2], Phi[3], Phi[4], Phi[7], Phi[9]};
         const bool ok = moments_frame3<R>(p, Psi, Tl, sq, Cv, rho, du, T1);
         pT = Tl;
 #pragma unroll
