@@ -81,9 +81,10 @@ __device__ __forceinline__ float vanleer_half(float a, float b)
     const float ab = a * b;
     return ab > 0.f ? ab * rcp_ftz(a + b) : 0.f;
 }
-// FP64: the reciprocal of a + b from the hardware's 20-bit seed and one third-order step
-// (r (1 + e + e^2), e = 1 - s r: the truncated Neumann series, error e^3 < 2^-57), and the test
-// ab > 0 on the sign and exponent bits; GB300 runs FP64 at 1/64 of the FP32 rate, and the
+// FP64: the quotient from the hardware's 20-bit reciprocal of a + b, one Newton step on it and one on the quotient
+// (q = q0 + r1 (ab - s q0), q0 = ab r0, r1 = r0 (2 - s r0)): the residual is exact to 2^-73 of ab and r1 to
+// 2^-38, so q is within 2^-57 of ab / s before its one rounding, as good as the division.  The test ab > 0 is
+// on the sign and exponent bits.  GB300 runs FP64 at 1/64 of the FP32 rate, and the
 // corrector evaluates this 64 times a pass in 2D and 384 times in 3D.  Where ab > 0, |a + b| is
 // above 2^-522, so the seed's flush of subnormals does not matter.
 __device__ __forceinline__ double vanleer_half(double a, double b)
@@ -91,9 +92,8 @@ __device__ __forceinline__ double vanleer_half(double a, double b)
     const double ab = a * b, s = a + b;
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(s));
-    const double e = fma(-s, r, 1.0);
-    r = fma(r, fma(e, e, e), r);
-    const double q = ab * r;
+    const double q0 = __dmul_rn(ab, r), r1 = fma(r, fma(-s, r, 1.0), r);
+    const double q = fma(fma(-s, q0, ab), r1, q0);
     // 0 < high word <= that of infinity: positive, not NaN
     return unsigned(__double2hiint(ab) - 1) < 0x7ff00000u ? q : 0.0;
 }
