@@ -166,7 +166,10 @@ pond_status pond_set_primitive(pond_state *s, const double *rho, const double *u
                                const double *uy, const double *p, int on_device);
 
 /* Enqueues n_steps time steps (Sec. III.B.4) on the state's stream and returns without
- * waiting.  The time step of each step comes from the CFL condition on the device. */
+ * waiting.  The time step of each step comes from the CFL condition on the device.
+ * Fewer than 32 finite-volume steps of a grid may be captured into a CUDA graph of the caller's and
+ * replayed, between other steps too; from the first capture on the state's steps run in place
+ * (the face and cell kernels). */
 pond_status pond_step(pond_state *s, int64_t n_steps);
 
 /* Same as pond_step, but launches every kernel individually with CUDA events around it on

@@ -119,6 +119,9 @@ struct pond_state {
     // planes; sl_parity counts the swaps
     int scheme = POND_FV;
     int sl_parity = 0;
+    // The caller has captured steps of this state into a graph of its own: grid steps run in place from
+    // then on (that graph holds the planes that were the state).  stale_graphs: ours are still the fused ones
+    bool in_place = false, stale_graphs = false;
     // batched tubes
     bool batch = false;
     int64_t n_tubes = 0, ncell = 0, nface = 0, steps_taken = 0;
@@ -445,11 +448,11 @@ void launch_fused(pond_state *s, pond::Params<D, R> &P)
 
 // the step runs fused: the tuner (or pond_set_variants) chose a fused variant and the step
 // is the plain one (the learned predictor, pair collection and the equilibration ablation
-// run the face and cell kernels)
+// run the face and cell kernels), and no graph of the caller's holds the planes
 template <int D, typename R>
 bool fused_step(const pond_state *s, bool collect)
 {
-    return s->tube_v > 0 && !s->learned && !collect && !s->equilibrate && s->scheme == POND_FV;
+    return s->tube_v > 0 && !s->in_place && !s->learned && !collect && !s->equilibrate && s->scheme == POND_FV;
 }
 
 template <int D, typename R>
@@ -482,6 +485,21 @@ void drop_graph(pond_state *s)
         if (s->graph[p]) cudaGraphDestroy(s->graph[p]);
         s->graph_exec[p] = nullptr;
         s->graph[p] = nullptr;
+    }
+}
+
+// Steps asked for while the caller captures the state's stream go into a graph that replays them on the
+// planes of today, any number of times and between other steps: from the first of them on the steps run in place.
+void note_capture(pond_state *s)
+{
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s->stream, &c) != cudaSuccess) cudaGetLastError();
+    if (c == cudaStreamCaptureStatusActive) {
+        s->stale_graphs = s->stale_graphs || !s->in_place;
+        s->in_place = true;
+    } else if (s->stale_graphs) {
+        drop_graph(s);   // (not while the caller captures)
+        s->stale_graphs = false;
     }
 }
 
@@ -1331,6 +1349,7 @@ pond_status pond_step(pond_state *s, int64_t n_steps)
 {
     if (pond_status st = check_state(s)) return st;
     if (n_steps < 0) return fail(POND_ERR_INVALID_ARG, "n_steps must be >= 0");
+    if (!s->batch && s->D != 3) note_capture(s);
     if (s->batch) return dispatch_batch(s, [&](auto r) { return batch_step<decltype(r)>(s, n_steps, nullptr); });
     if (s->D == 3) return s->prec == POND_FP32 ? step3_impl<float>(s, n_steps) : step3_impl<double>(s, n_steps);
     return dispatch(s, [&](auto d, auto r) { return step_impl<decltype(d)::value, decltype(r)>(s, n_steps); });
