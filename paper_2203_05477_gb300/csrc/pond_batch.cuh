@@ -303,11 +303,11 @@ tube_kernel(const TubeParams<R> P, int steps, int cur0)
                 for (int side = 0; side < 2; ++side) {
                     const int f = t + side;
                     const R dv[1] = {faceU[warp][f] - duc};
-                    add_face_flux<1, R, false, sizeof(R) == 8>(faceF[warp][f], faceG[warp][f], dv, faceT[warp][f], Tcr, invTc, rsqTc, 0,
+                    add_face_flux<1, R>(faceF[warp][f], faceG[warp][f], dv, faceT[warp][f], Tcr, invTc, rsqTc, 0,
                                         side ? sx : -sx, sqTc, ucr, H, G);
                 }
                 R Ho[4], Go[3], du[1], dT;
-                bool ok = cell_finish<1, R, sizeof(R) == 8>(H, G, invTc, sqTc, CvR, Ho, Go, du, dT);
+                bool ok = cell_finish<1, R>(H, G, invTc, sqTc, CvR, Ho, Go, du, dT);
                 const CellW un = fr_add(uc, du[0]);
                 const CellW Tn = fr_add(Tc, Tcr * dT);
                 const R unr = R(fr_lead(un)), Tnr = R(fr_lead(Tn));

@@ -2122,13 +2122,13 @@ cell_kernel(const Params<D, R> P)
 
 // ------------------------------------------------------------ fused step
 
-// Tile variants of the fused step: TX x TY cells per CTA, whose faces (TX+1) x TY along x
+// Tile variants of the fused D2Q16 step (D1Q4: pond_chunk.cuh): TX x TY cells per CTA, whose faces (TX+1) x TY along x
 // and TX x (TY+1) along y are all solved in the CTA (the faces on the tile's far edges are
 // also solved by the neighbouring tile), one thread per face; MINB CTAs per SM.
-template <int D, int TX_, int TY_, int MINB_>
+template <int TX_, int TY_, int MINB_>
 struct StepVariant {
-    static constexpr int TX = TX_, TY = D == 2 ? TY_ : 1, MINB = MINB_;
-    static constexpr int NXF = (TX + 1) * TY, NYF = D == 2 ? TX * (TY + 1) : 0, NF = NXF + NYF;
+    static constexpr int TX = TX_, TY = TY_, MINB = MINB_;
+    static constexpr int NXF = (TX + 1) * TY, NYF = TX * (TY + 1), NF = NXF + NYF;
     static constexpr int THREADS = ((NF + 31) / 32) * 32;
     static constexpr bool CHUNK = false;
 };
@@ -2136,11 +2136,11 @@ struct StepVariant {
 // the faces' populations (coefficients in the face frame, x, y order) and frames in shared
 // memory, one array per component (NF faces each), so that neighbouring threads touch
 // neighbouring words
-template <int D, typename R, int NF>
+template <typename R, int NF>
 struct FaceRecs {
-    R F[NCoef<D, 3>::value][NF];
-    R G[NCoef<D, 2>::value][NF];
-    typename FrameWords<R>::word fr[D + 1][NF];
+    R F[NCoef<2, 3>::value][NF];
+    R G[NCoef<2, 2>::value][NF];
+    typename FrameWords<R>::word fr[3][NF];
 };
 
 // One whole step (Sec. III.B.4) of a tile in one kernel: the CTA stages phi-bar-plus of the
@@ -2150,17 +2150,18 @@ struct FaceRecs {
 // and the face frames are read from sf, sg, sfr, xfr, yfr and written to their *_n copies,
 // so no CTA sees another's new values; faces on a tile's far edges are solved twice (by
 // both tiles) and written by their owner only.  Face populations never reach global memory.
-template <int D, typename R, typename V>
+template <typename R, typename V>
 __global__ void __launch_bounds__(V::THREADS, V::MINB)
-step_kernel(const Params<D, R> P)
+step_kernel(const Params<2, R> P)
 {
+    constexpr int D = 2;
     constexpr int TX = V::TX, TY = V::TY;
-    constexpr int BX = TX + 4, BY = D == 2 ? TY + 4 : 1;
+    constexpr int BX = TX + 4, BY = TY + 4;
     constexpr int NFC = NCoef<D, 3>::value, NGC = NCoef<D, 2>::value;
     using W = typename FrameWords<R>::word;
     __shared__ StagedCell<D, R> tile[BY * BX];
-    __shared__ StagedCell<D, R> tileT[D == 2 ? BY * BX : 1];
-    __shared__ FaceRecs<D, R, V::NF> frec;
+    __shared__ StagedCell<D, R> tileT[BY * BX];
+    __shared__ FaceRecs<R, V::NF> frec;
     __shared__ W utile[D];
 
     const Clock &K = *P.clock;
@@ -2172,21 +2173,16 @@ step_kernel(const Params<D, R> P)
     __syncthreads();
     for (int t = threadIdx.x; t < BX * BY; t += blockDim.x) {
         const int bx = t % BX, by = t / BX;
-        const long long ci = i0 - 2 + bx, cj = D == 2 ? j0 - 2 + by : 0;
-        if constexpr (D == 2) {
-            StagedCell<D, R> c;
-            load_cell_bar_plus<D, R>(P, ci, cj, cp, ce, utile, c);
-            tile[t] = c;
-            StagedCell<D, R> ct;
-            orient<D, 3, R>(c.A, ct.A, true);
-            orient<D, 2, R>(c.B, ct.B, true);
-            ct.du[0] = c.du[1];
-            ct.du[1] = c.du[0];
-            ct.T = c.T;
-            tileT[bx * BY + by] = ct;
-        } else {
-            load_cell_bar_plus<D, R>(P, ci, cj, cp, ce, utile, tile[t]);
-        }
+        StagedCell<D, R> c;
+        load_cell_bar_plus<D, R>(P, i0 - 2 + bx, j0 - 2 + by, cp, ce, utile, c);
+        tile[t] = c;
+        StagedCell<D, R> ct;
+        orient<D, 3, R>(c.A, ct.A, true);
+        orient<D, 2, R>(c.B, ct.B, true);
+        ct.du[0] = c.du[1];
+        ct.du[1] = c.du[0];
+        ct.T = c.T;
+        tileT[bx * BY + by] = ct;
     }
     __syncthreads();
 
@@ -2219,9 +2215,9 @@ step_kernel(const Params<D, R> P)
             cells.sn = 1;
             cells.st = BY;
         } else {
-            cells.base = &tile[(D == 2 ? int(fj - j0 + 2) * BX : 0) + int(fi - i0 + 2)];
+            cells.base = &tile[int(fj - j0 + 2) * BX + int(fi - i0 + 2)];
             cells.sn = 1;
-            cells.st = D == 2 ? BX : 0;
+            cells.st = BX;
         }
         const W *Frm = dir == 0 ? P.xfr : P.yfr;
         W *Frm_n = dir == 0 ? P.xfr_n : P.yfr_n;
@@ -2231,7 +2227,7 @@ step_kernel(const Params<D, R> P)
         for (int a = 0; a < D; ++a) uref[a] = Frm[a * nf + fidx];
         FaceCfg<R> cfg;
         cfg.h_dn = swap ? KC.h_dy : KC.h_dx;
-        cfg.h_dt = D == 2 ? (swap ? KC.h_dx : KC.h_dy) : R(0);
+        cfg.h_dt = swap ? KC.h_dx : KC.h_dy;
         cfg.Cv = P.Cv_r; cfg.tol = P.tol_r; cfg.wb = KC.wb; cfg.we = KC.we;
         cfg.limiter = P.limiter; cfg.max_iter = P.max_iter; cfg.fixed_iters = P.fixed_iters;
         const R Tp = R(fr_lead(Frm[D * nf + fidx]));
@@ -2239,10 +2235,8 @@ step_kernel(const Params<D, R> P)
         R dref[D], uabs[D];
         dref[0] = R(fr_rel(sel(uref, na), utile[na]));
         uabs[0] = R(fr_lead(sel(uref, na)));
-        if constexpr (D == 2) {
-            dref[1] = R(fr_rel(sel(uref, ta), utile[ta]));
-            uabs[1] = R(fr_lead(sel(uref, ta)));
-        }
+        dref[1] = R(fr_rel(sel(uref, ta), utile[ta]));
+        uabs[1] = R(fr_lead(sel(uref, ta)));
         FaceOut<D, R> o;
         solve_face<D, R>(cells, swap, dref, uabs, Tp, cfg, o);
         if (owned) {
@@ -2287,7 +2281,7 @@ step_kernel(const Params<D, R> P)
     if (t < TX * TY) do {
         const int tx = t % TX, ty = t / TX;
         const long long i = i0 + tx, j = j0 + ty;
-        if (i >= P.nx || (D == 2 && j >= P.ny)) break;
+        if (i >= P.nx || j >= P.ny) break;
         const long long c = j * P.nx + i;
         W uc[D];
 #pragma unroll
@@ -2320,11 +2314,9 @@ step_kernel(const Params<D, R> P)
         const R sx = KC.dt_dx;
         face_flux(ty * (TX + 1) + tx, 0, -sx, R(fr_lead(uc[0])));
         face_flux(ty * (TX + 1) + tx + 1, 0, sx, R(fr_lead(uc[0])));
-        if constexpr (D == 2) {
-            const R sy = KC.dt_dy;
-            face_flux(V::NXF + ty * TX + tx, 1, -sy, R(fr_lead(uc[1])));
-            face_flux(V::NXF + (ty + 1) * TX + tx, 1, sy, R(fr_lead(uc[1])));
-        }
+        const R sy = KC.dt_dy;
+        face_flux(V::NXF + ty * TX + tx, 1, -sy, R(fr_lead(uc[1])));
+        face_flux(V::NXF + (ty + 1) * TX + tx, 1, sy, R(fr_lead(uc[1])));
         R Ho[NFC], Go[NGC], du[D], dT;
         bool ok = cell_finish<D, R>(H, G, invTc, sqTc, Cv, Ho, Go, du, dT);
         W un[D];

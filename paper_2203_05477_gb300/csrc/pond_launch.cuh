@@ -117,11 +117,11 @@ template <int D, typename R>
 struct StepList;
 template <>
 struct StepList<2, float> {
-    using type = VList<StepVariant<2, 8, 8, 3>, StepVariant<2, 16, 4, 3>, StepVariant<2, 8, 4, 5>, StepVariant<2, 8, 8, 2>>;
+    using type = VList<StepVariant<8, 8, 3>, StepVariant<16, 4, 3>, StepVariant<8, 4, 5>, StepVariant<8, 8, 2>>;
 };
 template <>
 struct StepList<2, double> {
-    using type = VList<StepVariant<2, 8, 4, 2>, StepVariant<2, 4, 4, 4>>;
+    using type = VList<StepVariant<8, 4, 2>, StepVariant<4, 4, 4>>;
 };
 template <>
 struct StepList<1, float> {

@@ -94,8 +94,8 @@ void launch_step_one(const Params<D, R> &P, cudaStream_t st)
         const long long wave = (long long)(P.sms > 0 ? P.sms : 1) * V::MINB;
         chunk_step_kernel<R, V><<<unsigned(need < wave ? need : wave), V::THREADS, 0, st>>>(P);
     } else {
-        const dim3 g(unsigned((P.nx + V::TX - 1) / V::TX), D == 2 ? unsigned((P.ny + V::TY - 1) / V::TY) : 1u);
-        step_kernel<D, R, V><<<g, V::THREADS, 0, st>>>(P);
+        const dim3 g(unsigned((P.nx + V::TX - 1) / V::TX), unsigned((P.ny + V::TY - 1) / V::TY));
+        step_kernel<R, V><<<g, V::THREADS, 0, st>>>(P);
     }
 }
 template <int D, typename R, typename V, typename... Rest>

@@ -133,7 +133,6 @@ __device__ __forceinline__ FG<double> vanleer_half(FG<double> a, FG<double> b)
 }
 __device__ __forceinline__ FG<float> vminmod(FG<float> a, FG<float> b) { return {vminmod(Lane2{a.v}, Lane2{b.v}).v}; }
 __device__ __forceinline__ FG<double> vminmod(FG<double> a, FG<double> b) { return {vminmod(a.f, b.f), vminmod(a.g, b.g)}; }
-__device__ __forceinline__ FG<float> fgsel(bool c, FG<float> a, FG<float> b) { return {make_float2(c ? a.v.x : b.v.x, c ? a.v.y : b.v.y)}; }
 __device__ __forceinline__ FG<double> fgsel(bool c, FG<double> a, FG<double> b) { return {c ? a.f : b.f, c ? a.g : b.g}; }
 
 // ---- the regularized change of frame (Sec. II.C) in shift form
