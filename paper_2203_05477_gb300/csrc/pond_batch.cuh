@@ -22,9 +22,10 @@
 // Measured (GB300): 4096 tubes of 128 to 4096 cells in FP32 397 us a step (496 before a chunk's
 // loads were issued ahead of the previous chunk's faces, with offsets within a tube in 32 bits and
 // the chunk's state parked in shared memory meanwhile); bound by instruction issue, 1200 a cell.
-// FP64 tubes take the shift-form pass (pass1), which brought 136 tubes of 119 to 238 cells from
-// 343 to 226 us a step.  The FP32 pass stays node by node: where a corrector cycles
-// without converging its result depends on the rounding, and batches hold such faces.
+// Both precisions keep the node-by-node pass and round as they always have: where a corrector cycles
+// without converging its result depends on the rounding, and batches hold such faces (of 30 drawn FP64
+// batches the shift-form pass moved three by more than 4e-8, one by 5e-2).  FP64: 136 tubes of 119 to
+// 238 cells 341 us a step, 160 of 150 to 3000 cells 0.83 ms.
 #pragma once
 
 #include "pond_kernels.cuh"
@@ -78,7 +79,7 @@ tube_kernel(const TubeParams<R> P, int steps, int cur0)
 {
     constexpr int NW = THREADS / 32;
     constexpr int kStage = kTubeChunk + 4;
-    constexpr bool AHEAD = THREADS * MINB <= 512;   // 128 registers a thread or more
+    constexpr bool AHEAD = sizeof(R) == 4 && THREADS * MINB <= 512;   // 128 registers a thread or more
     using CellW = typename FrameWords<R>::word;
     __shared__ StagedCell<1, R> tile[NW][kStage];
     __shared__ R faceF[NW][kTubeChunk + 1][4];
@@ -156,7 +157,8 @@ tube_kernel(const TubeParams<R> P, int steps, int cur0)
         const R Cvh = CvR - R(0.5);
         const R *sf = P.sf[cur] + c_off, *sg = P.sg[cur] + c_off;
         const CellW *sfr = P.sfr[cur] + c_off;
-        // A chunk's loads are issued before the previous chunk is solved, but at 80 registers (AHEAD false), where they
+        // A chunk's loads are issued before the previous chunk is solved, but in FP64, where the arithmetic hides them
+        // (160 tubes of 150 to 3000 cells 0.85 ms ahead, 0.83 not), and at 80 registers (AHEAD false), where they
         // spill 272 B (us a step over 1000 steps, 256 threads / 3 CTAs: 176 ahead, 165 not; 256 / 2: 167 ahead,
         // 189 not; 128 / 4: 181 ahead, 240 not).  Lane l stages cell c0 - 2 + l (zero-gradient ends) and keeps its
         // state for the update below; lanes 0 and 1 also stage the right halo c0 + 30, c0 + 31.
@@ -241,7 +243,7 @@ tube_kernel(const TubeParams<R> P, int steps, int cur0)
                 const R dref[1] = {R(fr_rel(fu_c, utile))};
                 const R uabs[1] = {R(fr_lead(fu_c))};
                 FaceOut<1, R> o;
-                solve_face<1, R, false, 0, sizeof(R) == 8, sizeof(R) == 4 ? 1 : 0>(cells, false, dref, uabs, fT_c, cfg, o,
+                solve_face<1, R, false, 0, false, sizeof(R) == 4 ? 1 : 0>(cells, false, dref, uabs, fT_c, cfg, o,
                                                                FaceScratch{kept + (sizeof(R) == 4 ? threadIdx.x : 0), THREADS});
                 const bool owned = f < nc || k == L;
                 if (owned) {
@@ -303,11 +305,11 @@ tube_kernel(const TubeParams<R> P, int steps, int cur0)
                 for (int side = 0; side < 2; ++side) {
                     const int f = t + side;
                     const R dv[1] = {faceU[warp][f] - duc};
-                    add_face_flux<1, R>(faceF[warp][f], faceG[warp][f], dv, faceT[warp][f], Tcr, invTc, rsqTc, 0,
+                    add_face_flux<1, R, false, false>(faceF[warp][f], faceG[warp][f], dv, faceT[warp][f], Tcr, invTc, rsqTc, 0,
                                         side ? sx : -sx, sqTc, ucr, H, G);
                 }
                 R Ho[4], Go[3], du[1], dT;
-                bool ok = cell_finish<1, R>(H, G, invTc, sqTc, CvR, Ho, Go, du, dT);
+                bool ok = cell_finish<1, R, false>(H, G, invTc, sqTc, CvR, Ho, Go, du, dT);
                 const CellW un = fr_add(uc, du[0]);
                 const CellW Tn = fr_add(Tc, Tcr * dT);
                 const R unr = R(fr_lead(un)), Tnr = R(fr_lead(Tn));
@@ -409,9 +411,8 @@ tube_init_kernel(const TubeParams<R> P, int cur, const double *rho, const double
         const double ra = rho[a], rb = rho[b], ua = ux[a], ub = ux[b];
         const double Ea = p[a] * Cv + 0.5 * ra * ua * ua, Eb = p[b] * Cv + 0.5 * rb * ub * ub;
         const double r = 0.5 * (ra + rb), m = 0.5 * (ra * ua + rb * ub), E = 0.5 * (Ea + Eb);
-        const double u = m / r;
-        fr_store(P.fu[cur][f_off + k], u);
-        fr_store(P.fT[cur][f_off + k], (E - 0.5 * m * u) / (Cv * r));
+        fr_store(P.fu[cur][f_off + k], m / r);
+        fr_store(P.fT[cur][f_off + k], (E - 0.5 * m * m / r) / (Cv * r));
     }
     if (bad) { atomicAdd(&P.diag->nonphys, bad); atomicOr(&P.diag->flags, FLAG_NONPHYSICAL); any_bad = 1; }
 #pragma unroll
