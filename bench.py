@@ -439,7 +439,7 @@ D3_FACE_BYTES_PER_CELL = 140 + 3 * 32 + 456
 D3_CELL_BYTES_PER_CELL = 140 + 456 + 140
 # executed FP32 FLOP per face-pass of face3_kernel<float> and its tail (FFMA x 2 + FADD + FMUL, packed
 # forms x 2), counted by ncu on the 64^3 spherical explosion (profiles/face3_kernel_blast64_fp32.md)
-D3_FLOPS_PER_FACE_PASS = 17.4e3
+D3_FLOPS_PER_FACE_PASS = 17.6e3
 
 
 def bench_d3q64(args, n=128, steps=20, fp64_steps=3, rank=0):

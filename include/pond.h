@@ -141,7 +141,8 @@ typedef struct {
  * corrector of Sec. III.B.3 on the faces of all three axes (two tangential limited slopes
  * per face).  gamma <= 5/3 (Cv >= 3/2, Eq. geqPond).  The learned predictor and the
  * semi-Lagrangian scheme are D1Q4/D2Q16 features: options asking for them are refused
- * with POND_ERR_UNSUPPORTED.  On the returned state pond_step, pond_step_timed,
+ * with POND_ERR_UNSUPPORTED.  Device memory per cell: about 1.4 KB (FP64) or 0.9 KB (FP32), 8 B a face of it
+ * for the list of faces that take many passes.  On the returned state pond_step, pond_step_timed,
  * pond_sync, pond_get_state (coef_f [cells][20], coef_g [cells][10], frame [cells][4]:
  * ux, uy, uz, T; coefficient (r, s, t) at position (r+s+t)(r+s+t+1)(r+s+t+2)/6 +
  * (s+t)(s+t+1)/2 + t) and pond_destroy work as for the other grids; initial conditions,
@@ -174,7 +175,9 @@ pond_status pond_step(pond_state *s, int64_t n_steps);
 
 /* Same as pond_step, but launches every kernel individually with CUDA events around it on
  * the state's stream, waits, and adds the elapsed milliseconds of all face-corrector
- * launches to ms[0] and of all cell-update launches to ms[1] (ms: host array of 2). */
+ * launches to ms[0] and of all cell-update launches to ms[1] (ms: host array of 2).  A step that is one
+ * kernel (a batch's, the semi-Lagrangian one, a fused one: that of a 1D grid unless
+ * pond_set_variants chose the face and cell kernels) counts in ms[0] alone. */
 pond_status pond_step_timed(pond_state *s, int64_t n_steps, double ms[2]);
 
 /* Conserved fields rho, rho ux, rho uy, rho E per cell (Sec. II.B) into caller buffers

@@ -266,7 +266,8 @@ class Solver:
         _check(self.lib.pond_step(self.h, int(n)))
 
     def step_timed(self, n):
-        """n steps with every kernel timed by CUDA events on the stream: (face ms, cell ms)."""
+        """n steps with every kernel timed by CUDA events on the stream: (face ms, cell ms); a step that is
+        one kernel counts as face ms."""
         ms = np.zeros(2)
         _check(self.lib.pond_step_timed(self.h, int(n), _ptr(ms)))
         return float(ms[0]), float(ms[1])

@@ -11,7 +11,8 @@
 // FP32 steps are bit for bit those of the face and cell kernels (kRefFaces, Map1Written).
 //
 // Measured (GB300, us a step, before: face and cell kernels): FP32 4 M cells 201 (328), 200 000 cells 15.9
-// (26.7), 200 cells 7.6 (12.9, of which the serial step constants took 4); 16 warps per SM at 126 registers.
+// (26.7), 200 cells 7.6 (12.9, of which the serial step constants took 4); 74% of the issue slots with 16 warps per SM
+// (126 registers, no spills), 1240 thread instructions a cell.
 // 400 cells FP64 57 (155).  Short grids are bound by the chain of passes of the faces at a shock.
 #pragma once
 

@@ -27,10 +27,11 @@
 // Measured (GB300, us a launch; before: the best of the node-by-node tiles, that is 8 x 8 with
 // shared scratch in FP32 and 8 x 8 in FP64, and the 32 x 4 tile that was the default): FP32 quadrants
 // 1024^2 280 (328, default 446), shocked interface 1001 x 253 with minmod 93 (130, 186); FP64
-// quadrants 256^2 965 (3208), all with the tail kernel.  FP32 issues 143 M instructions where the node-by-node tile issued 252 M,
+// quadrants 256^2 981 (3208), all with the tail kernel.  FP32 issues 143 M instructions where the node-by-node tile issued 252 M,
 // at 49% of the issue slots with 12 warps per SM: a packed multiply-add with three different
 // register pairs takes four cycles of the register file (two with a repeated operand), the
-// dependent-instruction waits come next (1.6 of 6 cycles), then the loads around the pass.  Four CTAs
+// dependent-instruction waits come next (1.6 of 6 cycles), then the loads around the pass; 168 registers
+// spill 72 B.  Four CTAs
 // per SM would need 128 registers and spill 212 B (397 us at 8 x 16 cells); two leave the loads
 // exposed (318 us).
 #pragma once
@@ -413,6 +414,8 @@ template <typename R> constexpr int tail_ctas() { return sizeof(R) == 8 ? 2 : 4;
 // the CTA's own list 12 (1024^2 302 / 290 / 289 for 6 / 12 / 20).  FP64 (32 faces): a pass takes 64 cycles per
 // instruction however few lanes need it, so more go over, and all of them where the whole chip takes
 // them (49 x 583 / 64^2 / 256^2: 884 / 495 / 994 for 20, 718 / 375 / 969 for 31; smooth 300^2 2241 and 2266).
+// Smooth FP32 flows, two passes everywhere, pay for the list and are ahead of the node-by-node kernel all the
+// same (us a step, cells included): 40^2 26 (27), 100^2 28 (28), 200 x 150 32 (35), 300^2 60 (75), 1024^2 488 (702).
 template <typename R, int MODE>
 __host__ __device__ constexpr int coop_faces() { return sizeof(R) == 4 ? (chip_tail<R, MODE>() ? 40 : 12) : (chip_tail<R, MODE>() ? 31 : 20); }
 // how a face came to the list: to be passed again from its next frame, or after a pass that
@@ -1076,8 +1079,8 @@ lane_face_kernel(const Params<2, R> P)
 // of coop_tail, with lane q < 8 holding stencil cell q in registers and velocities relative to the face's
 // own predictor frame.  Faces that take many passes lie together (a shock crosses a few tiles), so a CTA's
 // own list keeps a few SMs busy while the others are done: the grid's list spreads them over the
-// chip.  Measured (GB300, us a launch of face and tail; before: each CTA its own list): FP64 quadrants 256^2 965
-// (1310), 64^2 365 (1007), 49 x 583 712 (1117), interface 401 x 201 1056 (1388), smooth 300^2 2260 (2222); FP32
+// chip.  Measured (GB300, us a launch of face and tail; before: each CTA its own list): FP64 quadrants 256^2 981
+// (1310), 64^2 367 (1007), 49 x 583 724 (1117), interface 401 x 201 1074 (1388), smooth 300^2 2292 (2222); FP32
 // quadrants 64^2 36 (81), 49 x 583 46 (76), 300^2 55 (107), 1024^2 280 (290), interface 1001 x 253 93 (110).
 // Two CTAs per SM in FP64 (three: 5% slower), four in FP32 (two: 7% slower at 1024^2).  Two warps a face, f and g
 // apart, halve the chain of a pass but cost twice the issue: FP64 850 at 49 x 583, 1105 at 256^2.

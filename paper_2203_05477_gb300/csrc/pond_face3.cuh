@@ -26,8 +26,8 @@
 // node-by-node kernel, where it is 0.93 times with these.
 //
 // Measured (GB300, ms a step's faces, before: the node-by-node kernel this one replaces): FP32 explosion
-// 64^3 0.74 (1.76), FP64 explosion 25 x 23 x 21 2.2 (15.3).  FP32 issues 52% of the slots with 12 warps
-// per SM (168 registers, no spills), the rest are dependent-instruction waits and the barrier;
+// 64^3 0.74 (1.76), FP64 explosion 25 x 23 x 21 2.2 (15.3).  FP32 issues 61% of the slots with 12 warps
+// per SM (167 registers, no spills; the tail 51 to 56%), the rest are dependent-instruction waits and the barrier;
 // FP64 is bound by its pipe (57% busy in the first pass, 65% in the tail).
 #pragma once
 

@@ -2424,7 +2424,8 @@ __device__ __forceinline__ void cell_conserved(const Params<D, R> &P, long long 
 }
 
 // Face predictor before the first step: frame of the pooled moments of the two cells.  Bound by the FP64
-// pipe, on which a division takes as long as nine multiply-adds; 32-bit face indices where they fit.
+// pipe, on which a division takes as long as nine multiply-adds; 32-bit face indices where they fit.  Setting 4 M
+// cells in FP32: 695 us (742 before the indices and the host's 1/dx).
 template <int D, typename R>
 __global__ void init_faces_kernel(const Params<D, R> P)
 {

@@ -17,9 +17,9 @@
 // took 80 transformations for 24 nodes, and evaluated every population at 16 points), and a
 // quarter of the pass is serial, which is what a small FP64 grid waits for.
 //
-// Measured (GB300, us a step; before: the thread per node): 500^2 FP32, two passes a node, 165 (329);
-// 100^2 FP64, three passes, 516 (2316); 31 x 51 FP64 260 (2156).  FP32 issues 1950 instructions a warp and pass at
-// 56% of the issue slots, with the shared-memory pipe at 64%: a lane reads 240 words of
+// Measured (GB300, us a step; before: the thread per node): 500^2 FP32, two passes a node, 164 (329);
+// 100^2 FP64, three passes, 516 (2316); 31 x 51 FP64 260 (2156).  FP32 issues 2000 instructions a warp and pass at
+// 61% of the issue slots, with the shared-memory pipe at 63% (1024^2: 63% and 68%): a lane reads 240 words of
 // the scratch a pass (320 before the writer formed the even and odd parts along x).  Two CTAs of
 // 64 nodes fill the shared memory; one node's scratch is 1.6 KB.  FP64 is bound by its pipe.
 #pragma once
