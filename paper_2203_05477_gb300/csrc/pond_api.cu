@@ -349,9 +349,14 @@ pond_status set_primitive_impl(pond_state *s, const double *rho, const double *u
     pond_status r = reset_clock(s);
     if (r != POND_OK) return r;
     pond::init_cells_kernel<D, R><<<blocks_for(n, 256), 256, 0, s->stream>>>(P, dr, dux, duy, dp, R(1.0 / P.dx), R(1.0 / P.dy));
-    const long long nf = P.nxf() + (D == 2 ? P.nyf() : 0);
-    pond::init_faces_kernel<D, R><<<blocks_for(nf, 256), 256, 0, s->stream>>>(P);
-    s->launches += 2;
+    s->launches += 1;
+    if (s->scheme != POND_SL) {
+        // (the semi-Lagrangian scheme keeps no face frames: its steps swap the state with the face planes, and after
+        // an odd number of them the planes that stand for the faces are the state's, shorter by a row)
+        const long long nf = P.nxf() + (D == 2 ? P.nyf() : 0);
+        pond::init_faces_kernel<D, R><<<blocks_for(nf, 256), 256, 0, s->stream>>>(P);
+        s->launches += 1;
+    }
     CUDA_TRY(cudaGetLastError());
     if (!on_device) CUDA_TRY(cudaStreamSynchronize(s->stream));
     return POND_OK;
