@@ -2120,6 +2120,23 @@ cell_kernel(const Params<D, R> P)
     reduce_rate_and_advance(P.clock, double(rate), true);
 }
 
+// Past t_end a step that changes buffers moves the state to the other ones as it is (the host swaps them
+// whatever the device does): planes of n words by the whole grid
+template <typename T>
+__device__ __forceinline__ void hold_planes(const T *from, T *to, long long n)
+{
+    const long long block = ((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    const long long stride = (long long)gridDim.x * gridDim.y * gridDim.z * blockDim.x;
+    for (long long i = block * blockDim.x + threadIdx.x; i < n; i += stride) to[i] = from[i];
+}
+template <int D, typename R>
+__device__ __forceinline__ void hold_state(const Params<D, R> &P, R *sf, R *sg, typename FrameWords<R>::word *sfr)
+{
+    hold_planes(P.sf, sf, Params<D, R>::NFS * P.ncell());
+    hold_planes(P.sg, sg, NCoef<D, 2>::value * P.ncell());
+    hold_planes(P.sfr, sfr, (D + 1) * P.ncell());
+}
+
 // ------------------------------------------------------------ fused step
 
 // Tile variants of the fused D2Q16 step (D1Q4: pond_chunk.cuh): TX x TY cells per CTA, whose faces (TX+1) x TY along x
@@ -2165,7 +2182,12 @@ step_kernel(const Params<2, R> P)
     __shared__ W utile[D];
 
     const Clock &K = *P.clock;
-    if (!(K.dt > 0.0)) return;  // t_end reached: the step is a no-op
+    if (!(K.dt > 0.0)) {
+        hold_state<2, R>(P, P.sf_n, P.sg_n, P.sfr_n);
+        hold_planes(P.xfr, P.xfr_n, (D + 1) * P.nxf());
+        hold_planes(P.yfr, P.yfr_n, (D + 1) * P.nyf());
+        return;
+    }
     const StepC<R> &KC = step_c<R>(K);
     const R cp = KC.cp, ce = KC.ce;
     const long long i0 = (long long)blockIdx.x * TX, j0 = (long long)blockIdx.y * TY;

@@ -73,7 +73,7 @@ sl_kernel(const Params<1, R> P)
     __shared__ SlCell1<R> tile[BX];
     __shared__ W utile[1];
     const Clock &K = *P.clock;
-    if (!(K.dt > 0.0)) return;
+    if (!(K.dt > 0.0)) return hold_state<1, R>(P, P.xf, P.xg, P.xfr);
     const StepC<R> &KC = step_c<R>(K);
     const long long n = P.ncell();
     const long long i0 = (long long)blockIdx.x * TX;

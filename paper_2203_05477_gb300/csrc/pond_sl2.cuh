@@ -118,7 +118,7 @@ sl2_kernel(const Params<2, R> P)
     __shared__ W utile[2];
     extern __shared__ __align__(16) unsigned char sl2_dyn[];
     const Clock &K = *P.clock;
-    if (!(K.dt > 0.0)) return;
+    if (!(K.dt > 0.0)) return hold_state<2, R>(P, P.xf, P.xg, P.xfr);
     const StepC<R> &KC = step_c<R>(K);
     const long long n = P.ncell();
     // gridDim.y ends at 65 535 tile rows; FP64 tiles, of two nodes a row, go on along z, a row past the grid updating
